@@ -220,8 +220,34 @@ static int span_lo_host(int s) { return (int)(int16_t)(s & 0xffff); }
 
 static int elem_size(int dtype) { return dtype == FIM_U8 ? 1 : (dtype == FIM_U16 ? 2 : 4); }
 
+// Vertical-slide table of a kernel (see Plan::vtab) for an ordinal image of row pitch SP whose box
+// starts at column xmin relative to the window of tile column 0. Returns its units (8 words each).
+static int fill_vtab(const fim_kernel* k, int SP, int xmin, int* tab) {
+    const int ncols = k->xmax - k->xmin + 1;
+    int cnt[2] = {0, 0};  // columns of even and odd box columns so far
+    auto put = [&](int parity, int top, int bot) {
+        int* t = tab + (cnt[parity] >> 1) * 8 + parity * 4 + (cnt[parity] & 1) * 2;
+        t[0] = top;
+        t[1] = bot;
+        ++cnt[parity];
+    };
+    for (int j = 0; j < ncols; ++j) {
+        const int dx = k->xmin + j;
+        put((dx - xmin) & 1, 2 * (k->ctop[j] * SP + dx), 2 * ((k->cbot[j] + 1) * SP + dx));
+    }
+    const int units = (std::max(cnt[0], cnt[1]) + 1) / 2;
+    for (int parity = 0; parity < 2; ++parity) {
+        // padding compares the list's last top entry with itself; a one-column kernel's empty list
+        // takes the pixel to the right of its only column's top entry (words of the same row)
+        const int off = cnt[parity] > 0 ? tab[((cnt[parity] - 1) >> 1) * 8 + parity * 4 + ((cnt[parity] - 1) & 1) * 2]
+                                        : tab[(1 - parity) * 4] + 2;
+        while (cnt[parity] < 2 * units) put(parity, off, off);
+    }
+    return units;
+}
+
 fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, const TileShape& ts, int smem_limit,
-                     Plan* p, int cta_threads, bool exact_ranks) {
+                     Plan* p, int cta_threads, bool exact_ranks, int rank_hi) {
     memset(p, 0, sizeof(*p));
     p->dtype = dtype;
     p->w = w;
@@ -237,9 +263,7 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
     p->G = ts.G;
     p->vthreads = 2 * ts.Tx * ts.RB;
     p->threads = std::max(p->vthreads, cta_threads);
-    // Scans are short in the small tiles of small kernels (4 groups per step) and long in the
-    // large tiles (8): measured on the 4096^2 photo-like workload, each within 2 % of the best.
-    p->scan_groups = p->vthreads < 1024 ? 4 : 8;
+    p->scan_groups = p->threads < 1024 ? 4 : 8;
     p->nwarps = p->threads / 32;
     if (p->threads > 1024 || p->threads % 32 != 0) return FIM_ERR_UNSUPPORTED;  // 2 x Tx x bands threads
     p->shape = k->shape;
@@ -254,11 +278,6 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
     p->rank = rank;
     p->nranks = 1;
     p->ranks[0] = rank;
-    // Small kernels: a warp's 32 chains drawn from every band even out the per-warp work of the
-    // vertical sweep (scan lengths follow the image content of a band); large kernels prefer the
-    // shorter per-step divergence of 32 adjacent columns of one band (measured on the 4096^2
-    // photo-like workload: mixing gains 4-13 % up to r = 16, loses 2-4 % from r = 32 on).
-    p->vmix = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1 <= 40 ? 1 : 0;
     p->S = ts.Tx + (k->xmax - k->xmin);
     p->SH = ts.Ty + (k->ymax - k->ymin);
     if (p->S > kMaxSide || p->SH > kMaxSide) return FIM_ERR_UNSUPPORTED;
@@ -280,39 +299,55 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
         p->frow[v] = (int)((uint32_t)(fl & 0xffff) | ((uint32_t)fr << 16));
         N += fr - fl + 1;
     }
-    // Footprints beyond 65535 pixels keep 16-bit ordinal ranks relative to the tile's feasible
-    // median ranks [rank, N - n + rank] (Fig. 10), which is all a pivot ever takes; callers whose
-    // targets vary per pixel or per kernel (exact_ranks) need N <= 65535.
+    // The ordinal image holds 16-bit ranks. Where the footprint has more than 32766 pixels they are
+    // relative to the tile's feasible target ranks [rank, N - n + rank_hi] (Fig. 10), which is all
+    // a pivot ever takes, if those fit signed 16 bits (the packed slides then take one compare
+    // instruction per pair of windows instead of three) or must (more than 65535 pixels); callers
+    // whose targets vary per pixel or per kernel (exact_ranks) need N <= 65535.
+    if (rank_hi < rank) rank_hi = rank;
     p->rank_base = 0;
-    if (N > 65535) {
-        if (exact_ranks || N > (1 << 20)) return FIM_ERR_UNSUPPORTED;
-        p->rank_base = std::max(0, rank - 1);
-        if (N - k->n + rank - p->rank_base > 65535) return FIM_ERR_UNSUPPORTED;
+    p->s16 = N <= kMaxSignedRank ? 1 : 0;
+    p->rel_max = p->s16 ? kMaxSignedRank : 65535;
+    if (!p->s16 && !exact_ranks && N <= (1 << 20)) {
+        const int base = std::max(0, rank - 1);
+        const int64_t top = N - k->n + rank_hi - base;  // the highest feasible rank, relative to base
+        if (top < kMaxSignedRank) {
+            p->rank_base = base;
+            p->s16 = 1;
+            p->rel_max = kMaxSignedRank;
+        } else if (N > 65535) {
+            if (top > 65535) return FIM_ERR_UNSUPPORTED;
+            p->rank_base = base;
+        }
+    } else if (N > 65535) {
+        return FIM_ERR_UNSUPPORTED;
     }
     p->N = (int)N;
-    // 8-bit coordinates (u - S/2, v - SH/2) reach (-128, -128), the mark of the padding entries,
-    // only at box position (0, 0) of a 256 x 256 box; they serve unless that corner belongs to the
-    // footprint (then it would be a real entry, and a member of some window).
+    // Omnigram coordinates are stored as (u - cx0, v - cy0). 8-bit ones reach (-128, -128), the mark
+    // of the padding entries, only at box position (0, 0) of a 256 x 256 box; they serve unless
+    // that corner belongs to the footprint (then it would be a real entry, and a member of some
+    // window). The disk test multiplies them by twice the window centre's coordinates as signed
+    // bytes (centres in [-63, 64]); 128-pixel tiles meet that with the origin at (S - 1) / 2,
+    // which boxes below 256 pixels allow.
     const bool corner = span_lo_host(p->frow[0]) == 0;
-    p->wide = (p->S > 256 || p->SH > 256 || (p->S == 256 && p->SH == 256 && corner)) ? 1 : 0;
-    p->cx0 = S / 2;
-    p->cy0 = p->SH / 2;
+    p->cx0 = S < 256 ? (S - 1) / 2 : S / 2;
+    p->cy0 = p->SH < 256 ? (p->SH - 1) / 2 : p->SH / 2;
+    const int px0 = -k->xmin - p->cx0, py0 = -k->ymin - p->cy0;  // the tile's first window centre
+    const bool far = p->shape == kShapeDisk &&
+                     (px0 < -63 || px0 + Tx - 1 > 64 || py0 < -63 || py0 + Ty - 1 > 64);
+    p->wide = (p->S > 256 || p->SH > 256 || (p->S == 256 && p->SH == 256 && corner) || far) ? 1 : 0;
     p->div_magic = (unsigned)(((1ull << 32) + (unsigned)S - 1) / (unsigned)S);
     int hs = 0;
-    while (((p->N - 1) >> hs) >= kSeedBins) ++hs;
+    const int rel_top = std::min(p->N - 1, p->rel_max);
+    while ((rel_top >> hs) >= kSeedBins) ++hs;
     p->hist_shift = hs;
     // Seeds: the omnigram walk reads about N/2 entries, the histogram n pixels with a shared-memory
     // atomic each; the walk wins where the footprint is small against the kernel (measured on the
     // 4096^2 photo-like workload: walk +1 % at r = 64, +8 % at r = 96; histogram ahead up to r = 48).
     p->seed_mode = p->N < 4 * p->n ? kSeedWalk : kSeedHistogram;
-    if (p->rank_base > 0) p->seed_mode = kSeedWalk;  // the histogram bins the ordinal image's ranks
     if (const char* e = getenv("FIM_SEEDS"))  // experiments: 0 histogram, 1 walk, 2 count at the middle
         if (*e >= '0' && *e <= '2' && e[1] == 0) p->seed_mode = *e - '0';
-    for (int j = 0; j < p->ncols; ++j) {
-        const int dx = k->xmin + j;
-        p->vtab[2 * j] = k->ctop[j] * SP + dx;
-        p->vtab[2 * j + 1] = (k->cbot[j] + 1) * SP + dx;
-    }
+    p->vunits = fill_vtab(k, SP, k->xmin, p->vtab);
     for (int i = 0; i < p->nrows; ++i) {
         const int dy = k->ymin + i;
         p->htab[2 * i] = dy * SP + k->rlo[i];
@@ -352,11 +387,11 @@ fim_status plan_stage_model(Plan* p, int smem_limit) {
 }
 
 fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
-    const int Tx = p->Tx, Ty = p->Ty, SP = p->SP;
+    const int Tx = p->Tx, SP = p->SP;
     const size_t omb = p->wide ? 4 : 2;      // omnigram entry / position bytes
-    const size_t om_bytes = align16((size_t)p->N * omb);
+    const size_t om_bytes = ((size_t)p->N * omb + 63) & ~(size_t)63;  // whole 64-byte blocks
     const size_t ord_bytes = align16((size_t)SP * p->SH * 2);
-    const size_t med_bytes = align16((size_t)Tx * Ty * 2);
+    const size_t med_bytes = align16((size_t)p->RB * Tx * 2);
     // one coarse histogram per concurrently solved seed; seeds that walk the omnigram need none
     // (the learned seeds keep one histogram's room for the MLP's shared pre-activations)
     const size_t shist_bytes =
@@ -367,16 +402,19 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
         *field = (int)tab;
         tab += align16(bytes);
     };
-    take_tab(&p->off_vtab, (size_t)p->ncols * 8);
+    take_tab(&p->off_vtab, (size_t)p->vunits * 32);
     take_tab(&p->off_htab, (size_t)p->nrows * 8);
     take_tab(&p->off_spans, (size_t)p->nrows * 4);
     take_tab(&p->off_frow, (size_t)p->SH * 4);
+    p->off_test = -1;
+    if (p->shape == kShapeSpans) take_tab(&p->off_test, (size_t)(p->nrows + 1) * kSpanCopies * 4);
     p->off_model = -1;
     if (stage_model) take_tab(&p->off_model, (size_t)kMlpParams * 2);
     if (p->xtab_words > 0) take_tab(&p->off_xtab, (size_t)p->xtab_words * 4);
     p->tab_bytes = (int)tab;  // everything from here on belongs to one tile group
     p->off_misc = (int)tab;
     tab += 256;
+    tab = (tab + 63) & ~(size_t)63;  // the omnigram, first after the tables, is read in 64-byte blocks
     auto gloc = [](size_t off) { return -(int)off - 1; };
     p->loc_bins = p->loc_keys = p->loc_a = p->loc_b = p->loc_hist = 0;
     p->loc_dig = -1;
@@ -548,8 +586,8 @@ static bool parse_tile_env(TileShape* ts) {
 
 fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape* ts, int w, int h,
                        int cta_threads, bool exact_ranks) {
-    static const TileShape cands[] = {{32, 32, 2, 1}, {32, 32, 4, 1}, {64, 128, 8, 2}, {64, 64, 8, 2},
-                                      {32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
+    static const TileShape cands[] = {{32, 32, 2, 1}, {32, 32, 4, 1}, {64, 128, 8, 2}, {64, 120, 8, 2},
+                                      {64, 64, 8, 2}, {32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
     TileShape forced;
     if (parse_tile_env(&forced)) {  // explicit override (experiments, tuning)
         Plan* p = new (std::nothrow) Plan;
@@ -581,7 +619,7 @@ fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape
     // across: the same tiles with four bands; up to 64 across: 64x64 tiles in 1024-thread CTAs;
     // beyond: taller 64x128 tiles, which halve the seed and seed-row work per pixel.
     const int extent = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1;
-    const int first = extent <= 33 ? 0 : (extent <= 45 ? 1 : (extent >= 65 ? 2 : 3));
+    const int first = extent <= 33 ? 0 : (extent <= 45 ? 1 : (extent >= 65 ? 2 : 4));
     // Beyond the first valid shape, two measured exceptions (4096^2 photo-like u16, 4096^2 u8,
     // 8192^2 f32):
     // (1) where its omnigram spills to global scratch, a later shape of at least 64x64 whose
@@ -911,8 +949,7 @@ fim_status fim_percentiles(const void* in, void* const* outs, const double* perc
         rmax = std::max(rmax, ranks[i]);
     }
     // offset ranks (large footprints) must resolve every target's feasible ranks
-    s = make_plan(k, dtype, rmin, w, h, ts, smem_limit, p);
-    if (s == FIM_OK && p->N > 65535 && p->N - k->n + rmax - p->rank_base > 65535) s = FIM_ERR_UNSUPPORTED;
+    s = make_plan(k, dtype, rmin, w, h, ts, smem_limit, p, 0, false, rmax);
     if (s == FIM_OK) {
         p->in = in;
         p->out = outs[0];
@@ -964,12 +1001,12 @@ fim_status fim_median_radii(const void* in, void* const* outs, const fim_kernel*
         const int SP = p->SP, SH = p->SH, Tx = p->Tx, Ty = p->Ty;
         for (int q = 0; q < count; ++q) {
             const fim_kernel* k = kernels[order[q]];
-            const int nrows = k->ymax - k->ymin + 1, ncols = k->xmax - k->xmin + 1;
+            const int nrows = k->ymax - k->ymin + 1;
+            while (xt.size() & 3) xt.push_back(0);  // the vertical-slide lists are read 16 bytes at a time
             rel_v[q] = (int)xt.size();
-            for (int j = 0; j < ncols; ++j) {
-                xt.push_back(k->ctop[j] * SP + k->xmin + j);
-                xt.push_back((k->cbot[j] + 1) * SP + k->xmin + j);
-            }
+            xt.resize(xt.size() + 2 * (size_t)(kMaxExtent + 4));
+            p->q_vunits[q] = fill_vtab(k, SP, p->xmin, xt.data() + rel_v[q]);
+            xt.resize(rel_v[q] + 8 * (size_t)p->q_vunits[q]);
             rel_h[q] = (int)xt.size();
             for (int i = 0; i < nrows; ++i) {
                 xt.push_back((k->ymin + i) * SP + k->rlo[i]);
@@ -992,17 +1029,14 @@ fim_status fim_median_radii(const void* in, void* const* outs, const fim_kernel*
                 xt.push_back((int)((uint32_t)(lo & 0xffff) | ((uint32_t)hi << 16)));
                 nq += hi - lo + 1;
             }
-            if (xt.size() & 1) xt.push_back(0);  // the next disk's int2 tables stay 8-byte aligned
             p->q_r2[q] = (int)k->r2;
             p->q_n[q] = k->n;
             p->q_ymin[q] = k->ymin;
             p->q_nrows[q] = nrows;
-            p->q_ncols[q] = ncols;
             p->q_N[q] = (int)nq;
             int hs = 0;
             while (((nq - 1) >> hs) >= kSeedBins) ++hs;
             p->q_hshift[q] = hs;
-            p->q_vmix[q] = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1 <= 40 ? 1 : 0;
             p->ranks[q] = (k->n - 1) / 2;
             p->outs[q] = outs[order[q]];
         }

@@ -18,6 +18,8 @@ constexpr int kMaxExtent = 264;   // kernel rows / columns held in a plan (>= FI
 constexpr int kMaxSide = 400;     // bounding-box rows of a tile footprint held in a plan
 constexpr int kSortBins = 256;    // 8-bit radix digits
 constexpr int kSeedBins = 256;    // coarse histogram bins of a seed solve
+constexpr int kSpanCopies = 8;    // copies of the span test's table, one per lane modulo 8
+constexpr int kMaxSignedRank = 32766;  // ordinal-image ranks the packed 16-bit compares take as signed
 
 enum Shape : int { kShapeDisk = 0, kShapeSpans = 1 };
 
@@ -81,8 +83,7 @@ struct Plan {
     int Tx, Ty, txshift, RB, G;
     int threads, nwarps;    // CTA size (all cooperative loops and per-warp buffers)
     int vthreads;           // 2*Tx*RB: threads of the vertical sweep (the first ones of the CTA)
-    int vmix;               // 1: the lanes of a vertical-sweep warp take their columns from all bands
-    int scan_groups;        // 128-bit omnigram groups a vertical-sweep lane tests per scan step
+    int scan_groups;        // kernel set: 8 the 1024-thread CTAs', 4 the smaller ones' (fim_tile_k4.cu)
     int S, SH;              // footprint bounding box (columns, rows)
     int SP;                 // row pitch (elements) of the ordinal image; SP/2 is odd
     int tiles_x, tiles_y;
@@ -90,6 +91,7 @@ struct Plan {
     int shape;
     int r2;                 // disk: dx^2 + dy^2 <= r2
     int xmin, xmax, ymin, ymax, nrows, ncols;
+    int vunits;             // vertical-slide table: units of two even and two odd columns (see vtab)
     int n;                  // taps
     int rank;               // target 0-based rank ((n-1)/2 for the median)
     int nranks;             // extras kernels: target ranks served by one ordinal transform (1..kMaxRanks)
@@ -99,16 +101,18 @@ struct Plan {
     // nested in the plan's kernel (which sets the footprint); its tables sit in shared memory
     int multi;                          // 1: the q_ arrays below give each target's kernel
     int q_vtab[kMaxRanks], q_htab[kMaxRanks], q_spans[kMaxRanks];  // shared-memory byte offsets
-    int q_r2[kMaxRanks], q_n[kMaxRanks], q_ymin[kMaxRanks], q_nrows[kMaxRanks], q_ncols[kMaxRanks];
+    int q_r2[kMaxRanks], q_n[kMaxRanks], q_ymin[kMaxRanks], q_nrows[kMaxRanks];
     int q_frow[kMaxRanks];              // shared-memory byte offset of each disk's footprint rows
     int q_N[kMaxRanks], q_hshift[kMaxRanks];  // its footprint size and seed-histogram shift
-    int q_vmix[kMaxRanks];              // its vertical-sweep lane mixing (as `vmix` for its own plan)
+    int q_vunits[kMaxRanks];          // its vertical-slide table's units
     const int* xtab;                    // device: those tables, copied to shared memory at off_xtab
     int xtab_words;                     // their length in 32-bit words
     int off_xtab;
     // footprint
     int N;                  // pixels in the rounded-rectangle footprint
-    int rank_base;          // the ordinal image and the medians hold rank - rank_base (16 bits)
+    int rank_base;          // the ordinal image and the medians hold rank - rank_base,
+    int rel_max;            //   clamped to [0, rel_max]
+    int s16;                // 1: those ranks fit signed 16 bits (rel_max <= 32766)
     int cx0, cy0;           // omnigram coordinates are stored as (u - cx0, v - cy0), int8 each
     unsigned div_magic;     // ceil(2^32 / S): v = umulhi(pos, magic) = pos / S for pos < 2^32 / S (radix path)
     int hist_shift;         // seed histogram: bin = rank >> hist_shift
@@ -133,6 +137,7 @@ struct Plan {
     // Array placement. A location >= 0 is a byte offset into dynamic shared memory; a location
     // < 0 is -(offset + 1) into the CTA's slice of global scratch.
     int off_vtab, off_htab, off_spans, off_frow;   // tables (shared memory, whole kernel)
+    int off_test;                                   // span test words, or -1 (disks)
     int off_model;                                  // bracket MLP parameters in shared memory, or -1
     int tab_bytes;                                  // the tables' extent; a tile group's partition follows
     int off_misc;                                   // 64 words of scan scratch (per group)
@@ -142,7 +147,7 @@ struct Plan {
     int loc_bins;                                   // counting sorts: bins
     int loc_keys, loc_a, loc_b, loc_hist;           // radix sort: keys, ping-pong lists, histograms
     int loc_dig;                                    // radix sort with keys in global scratch: digit bytes (-1: none)
-    int loc_ord, loc_med, loc_shist;                // solve: ordinal image, medians, seed histograms
+    int loc_ord, loc_med, loc_shist;                // solve: ordinal image, seed rows' medians, seed histograms
     int smem_bytes;
     long long scratch_per_cta;  // bytes of global scratch per resident CTA (multiple of 256)
     // persistent grid
@@ -151,7 +156,11 @@ struct Plan {
     unsigned char* scratch;     // header (256 B: tile counter) + grid * scratch_per_cta
     // tables (copied to shared memory at kernel start)
     int frow[kMaxSide];                   // footprint row v covers u in [lo, hi]: lo | hi << 16
-    int vtab[2 * kMaxExtent];             // per column j: top*SP + dx, (bot+1)*SP + dx
+    // Vertical slides: per kernel column the byte offsets of its top entry and of the one below its
+    // bottom, from the window centre in the ordinal image. Columns whose box column is even for an
+    // even window column, two by two, alternate with the odd ones; the shorter list is padded with
+    // entries that compare a pixel with itself.
+    int vtab[2 * (kMaxExtent + 4)];
     int htab[2 * kMaxExtent];             // per row i: dy*SP + lo, dy*SP + hi + 1
     int spans[kMaxExtent];                // per row i: (lo & 0xffff) | (hi << 16)
     // tensor map of the input image for the footprint copies (valid when use_tma)
@@ -204,9 +213,9 @@ fim_status release_scratch();
 int device_sm_count();
 // exact_ranks: the plan's targets vary per pixel or per kernel, so its ordinal image must hold
 // exact ranks (footprints up to 65535 pixels); otherwise larger footprints hold ranks relative to
-// the feasible median ranks of `rank`.
+// the feasible ranks of the targets `rank` .. `rank_hi` (-1: `rank` alone).
 fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, const TileShape& ts, int smem_limit,
-                     Plan* p, int cta_threads = 0, bool exact_ranks = false);
+                     Plan* p, int cta_threads = 0, bool exact_ranks = false, int rank_hi = -1);
 // Re-lays out a plan whose model is set so that the bracket MLP's parameters are staged in
 // shared memory; keeps them in device memory (off_model = -1) when they do not fit.
 fim_status plan_stage_model(Plan* p, int smem_limit);

@@ -52,11 +52,11 @@ fim_status workspace_address(unsigned char** out) {
 // fits the fixed array (per-CTA buffers of large kernels times the resident CTAs). Trial plans
 // and the chosen one are built in the caller's storage.
 fim_status pick_plan(const fim_kernel* k, int dtype, int w, int h, int limit, fim::Plan* plan) {
-    static const fim::TileShape cands[] = {{32, 32, 2, 1}, {32, 32, 4, 1}, {64, 128, 8, 2}, {64, 64, 8, 2},
-                                           {32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
+    static const fim::TileShape cands[] = {{32, 32, 2, 1}, {32, 32, 4, 1}, {64, 128, 8, 2}, {64, 120, 8, 2},
+                                           {64, 64, 8, 2}, {32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
     const int ncands = (int)(sizeof(cands) / sizeof(cands[0]));
     const int extent = (k->xmax - k->xmin > k->ymax - k->ymin ? k->xmax - k->xmin : k->ymax - k->ymin) + 1;
-    const int first = extent <= 33 ? 0 : (extent <= 45 ? 1 : (extent >= 65 ? 2 : 3));
+    const int first = extent <= 33 ? 0 : (extent <= 45 ? 1 : (extent >= 65 ? 2 : 4));
     auto valid = [&](int i) {
         return fim::make_plan(k, dtype, (k->n - 1) / 2, w, h, cands[i], limit, plan) == FIM_OK &&
                plan->smem_bytes <= limit &&

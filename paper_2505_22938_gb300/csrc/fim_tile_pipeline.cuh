@@ -19,9 +19,9 @@
 //   4. seed rows       - one warp per (seed, direction) slides the window left/right; lanes
 //                        split the kernel rows and reduce the count change (Sec. 3.3 step 4).
 //   5. vertical sweep  - one thread per (column, band, direction) slides its window up or
-//                        down (Fig. 7) and refines it by scanning Omega itself, K 128-bit
-//                        groups per step; the last few lanes of a warp hand their long scans to
-//                        warp ballots (Sec. 4.1, Eq. 2).
+//                        down (Fig. 7), sharing packed compares with its neighbour's window, and
+//                        refines it by scanning Omega itself in 64-byte blocks; the last few
+//                        lanes of a warp hand very long scans to warp ballots (Sec. 4.1, Eq. 2).
 //   6. output          - out = C[m] through the omnigram: the input value at Omega[m].
 // Pivots are exact previous medians (Huang's choice, Sec. 3.1): after each solve the count
 // below the pivot is exactly the target rank, and a slide only adds the change.
@@ -148,7 +148,7 @@ struct Grp {
 // stores.
 __device__ __forceinline__ void stamp(const Plan& P, int tile, int phase, const Grp& G) {
     if (P.phase_clock != nullptr && G.tid == 0 && tile < P.phase_tiles) {
-        extern __shared__ __align__(16) unsigned char smem_base[];
+        extern __shared__ __align__(128) unsigned char smem_base[];
         unsigned long long* st = reinterpret_cast<unsigned long long*>(smem_base + G.shift + P.off_misc + 48 * 4);
         st[phase] = clock64();
         if (phase == 7)
@@ -159,92 +159,184 @@ __device__ __forceinline__ void stamp(const Plan& P, int tile, int phase, const 
 __device__ __forceinline__ int span_lo(int s) { return (int)(int16_t)(s & 0xffff); }
 __device__ __forceinline__ int span_hi(int s) { return s >> 16; }
 
-// Region membership of one omnigram entry (Eq. 2); (px, py) is the window centre in the
-// entry's coordinate frame.
+// The kernel as the membership tests need it (Eq. 2, Eq. 3).
 template <int SHAPE, int W>
 struct Member;
 
 template <int W>
 struct Member<kShapeDisk, W> {
-    int r2;
-    __device__ __forceinline__ bool operator()(uint32_t e, int px, int py) const {
-        const int dx = Loc<W>::x(e) - px;
-        const int dy = Loc<W>::y(e) - py;
-        return dx * dx + dy * dy <= r2;   // Eq. 3 on the lattice
-    }
+    int r2;  // dx^2 + dy^2 <= r2
 };
 
 template <int W>
 struct Member<kShapeSpans, W> {
-    const int* spans;  // shared memory, per kernel row: lo | hi << 16
-    int ymin, nrows;
-    __device__ __forceinline__ bool operator()(uint32_t e, int px, int py) const {
-        const int i = Loc<W>::y(e) - py - ymin;
-        if ((unsigned)i >= (unsigned)nrows) return false;
-        const int s = spans[i];
-        const int dx = Loc<W>::x(e) - px;
-        return dx >= span_lo(s) && dx <= span_hi(s);
-    }
+    const uint32_t* test;  // shared memory: the rows' test words (see WordTest)
+    int xmin, ymin, nrows;
 };
 
-// Membership of the omnigram entries held in one 32-bit word, for a fixed window: bit k is
-// entry k of the word (two 16-bit entries, or one 32-bit entry).
+// Membership of the omnigram entries held in one 32-bit word (two 16-bit entries, or one 32-bit
+// entry), for a fixed window whose centre (px, py) is given in the entries' coordinate frame:
+// bit k of operator() is entry k of the word.
 template <int SHAPE, int W>
-struct WordTest {
-    Member<SHAPE, W> m;
-    int px, py;
-    __device__ __forceinline__ void init(const Member<SHAPE, W>& mm, int x, int y) {
-        m = mm;
-        px = x;
-        py = y;
-    }
-    __device__ __forceinline__ uint32_t operator()(uint32_t w) const {
-        if constexpr (W == 0)
-            return (uint32_t)m(w & 0xffffu, px, py) | ((uint32_t)m(w >> 16, px, py) << 1);
-        else
-            return (uint32_t)m(w, px, py);
-    }
-};
+struct WordTest;
 
-// Disk with 8-bit coordinates: (x-px)^2 + (y-py)^2 <= r2 is evaluated as
-// x^2 + y^2 - 2(x px + y py) <= r2 - px^2 - py^2 with byte dot products on the packed pair.
+// Disk with 8-bit coordinates: (x-px)^2 + (y-py)^2 <= r2 is evaluated as the sign of
+// x^2 + y^2 - 2(x px + y py) + px^2 + py^2 - r2 - 1, two byte dot products per entry on the packed
+// pair. The plan keeps -2px and -2py in a signed byte (px, py in [-63, 64]).
 template <>
 struct WordTest<kShapeDisk, 0> {
-    int R;
-    int plo, phi;  // (px, py, 0, 0) and (0, 0, px, py) as signed bytes
+    int nR;        // px^2 + py^2 - r2 - 1
+    int plo, phi;  // (-2px, -2py, 0, 0) and (0, 0, -2px, -2py) as signed bytes
     __device__ __forceinline__ void init(const Member<kShapeDisk, 0>& mm, int px, int py) {
-        R = mm.r2 - px * px - py * py;
-        const uint32_t b = (uint32_t)(px & 0xff) | ((uint32_t)(py & 0xff) << 8);
+        nR = px * px + py * py - mm.r2 - 1;
+        const uint32_t b = (uint32_t)((-2 * px) & 0xff) | ((uint32_t)((-2 * py) & 0xff) << 8);
         plo = (int)b;
         phi = (int)(b << 16);
     }
+    // negative iff the low / high entry of the word is a member
+    __device__ __forceinline__ int lo(uint32_t w) const {
+        return __dp4a((int)w, plo, __dp4a((int)(w & 0xffffu), (int)w, nR));
+    }
+    __device__ __forceinline__ int hi(uint32_t w) const {
+        return __dp4a((int)w, phi, __dp4a((int)(w & 0xffff0000u), (int)w, nR));
+    }
     __device__ __forceinline__ uint32_t operator()(uint32_t w) const {
-        const int sq = __dp4a((int)w, (int)w, 0);
-        const int sq0 = __dp4a((int)(w & 0xffffu), (int)w, 0);
-        const int t0 = sq0 - 2 * __dp4a((int)w, plo, 0);
-        const int t1 = (sq - sq0) - 2 * __dp4a((int)w, phi, 0);
-        return (uint32_t)(t0 <= R) | ((uint32_t)(t1 <= R) << 1);
+        return ((uint32_t)lo(w) >> 31) | (((uint32_t)hi(w) >> 31) << 1);
     }
 };
 
-// Exact selection by ballot scans of the omnigram (Sec. 4.1, Sec. 4.2).
-// Given a pivot rank p and c = #{window members with rank < p}, returns the rank m of the
-// window element with window-rank `target`. All 32 lanes pass the same arguments and get
-// the same result; -1 means the counts were inconsistent (never expected).
-template <class E, class M>
-__device__ __forceinline__ int ballot_select(const E* __restrict__ om, int N, int p, int c, int target, int px,
-                                             int py, const M& member) {
+// Any convex shape. A kernel row's columns [lo, hi] (counted from the kernel's first column, plus
+// 256) stand in one word (0x8000 - lo, 0x7fff - hi): added to the entry's column in both halves,
+// bit 31 says "from lo on" and bit 15 "past hi", so that an entry takes two dot products that pick
+// its coordinates, a row clamp, a table load, a multiply-add and two bit operations. Row nrows
+// stands for every row outside the kernel and holds no column. The entries a warp tests at once
+// lie in unrelated rows: eight copies of the table, side by side for the lanes modulo 8, halve the
+// bank conflicts of their loads (3.5 -> 2.1 wavefronts on random rows).
+template <int W>
+struct WordTest<kShapeSpans, W> {
+    const uint32_t* test;
+    int cx, cy, nrows;
+    __device__ __forceinline__ void init(const Member<kShapeSpans, W>& mm, int px, int py) {
+        test = mm.test + (threadIdx.x & (kSpanCopies - 1));
+        cx = 256 - mm.xmin - px;
+        cy = -mm.ymin - py;
+        nrows = mm.nrows;
+    }
+    __device__ __forceinline__ int column(int x, int y) const {
+        const uint32_t e = (uint32_t)x * 65537u + test[min((uint32_t)y, (uint32_t)nrows) * kSpanCopies];
+        return (int)(e & ~(e << 16));
+    }
+    // negative iff the low / high entry of the word (W = 0), or the word (W = 1), is a member
+    __device__ __forceinline__ int lo(uint32_t w) const {
+        if constexpr (W == 0) return column(__dp4a((int)w, 0x00000001, cx), __dp4a((int)w, 0x00000100, cy));
+        else return column(__dp2a_lo((int)w, 0x0001, cx), __dp2a_lo((int)w, 0x0100, cy));
+    }
+    __device__ __forceinline__ int hi(uint32_t w) const {
+        return column(__dp4a((int)w, 0x00010000, cx), __dp4a((int)w, 0x01000000, cy));
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t w) const {
+        if constexpr (W == 0) return ((uint32_t)lo(w) >> 31) | (((uint32_t)hi(w) >> 31) << 1);
+        else return (uint32_t)lo(w) >> 31;
+    }
+};
+
+// A disk with 16-bit coordinates.
+template <>
+struct WordTest<kShapeDisk, 1> {
+    int r2, px, py;
+    __device__ __forceinline__ void init(const Member<kShapeDisk, 1>& mm, int x, int y) {
+        r2 = mm.r2;
+        px = x;
+        py = y;
+    }
+    __device__ __forceinline__ int lo(uint32_t w) const {  // negative iff the entry is a member
+        const int dx = Loc<1>::x(w) - px, dy = Loc<1>::y(w) - py;
+        return dx * dx + dy * dy - r2 - 1;
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t w) const { return (uint32_t)lo(w) >> 31; }
+};
+
+// Appends the word's membership bits below `mask` (mask moves up by the entries of a word): the
+// sign of each entry's test shifts straight in, one funnel shift per entry.
+template <int SHAPE, int W>
+__device__ __forceinline__ uint32_t push_word(uint32_t mask, const WordTest<SHAPE, W>& wt, uint32_t w) {
+    if constexpr (W == 0) mask = __funnelshift_l((uint32_t)wt.hi(w), mask, 1);
+    return __funnelshift_l((uint32_t)wt.lo(w), mask, 1);
+}
+
+// Membership of the entries of one 64-byte block of the omnigram (32 entries of 16 bits, 16 of 32
+// bits): bit k is entry k. Every lane reads its own block. All lanes starting with their block's
+// first 16 bytes would meet in two of the eight bank quads per load; lane l instead reads its
+// quads in the order k ^ (l & 3), so that a load's eight lanes cover four quads of one half, and
+// the order is undone when the four part masks are joined (measured on random blocks: 13.7
+// cycles per 128-bit load unordered). The four parts are also independent shift chains.
+template <int SHAPE, int W>
+__device__ __forceinline__ uint32_t block_mask(const uint4* om128, int b, const WordTest<SHAPE, W>& wt) {
+    const int l3 = threadIdx.x & 3;
+    const uint4* blk = om128 + 4 * b;
+    uint4 q[4];
+    uint32_t part[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q[k] = blk[k ^ l3];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t m = push_word(0u, wt, q[k].w);
+        m = push_word(m, wt, q[k].z);
+        m = push_word(m, wt, q[k].y);
+        part[k] = push_word(m, wt, q[k].x);
+    }
+    if constexpr (W == 0) {  // one byte per part
+        const uint32_t s0 = l3 & 1 ? 0x1104u : 0x1140u, s1 = l3 & 2 ? 0x1054u : 0x5410u;
+        return __byte_perm(__byte_perm(part[0], part[1], s0), __byte_perm(part[2], part[3], s0), s1);
+    } else {
+        uint32_t m = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) m |= part[k] << (4 * (k ^ l3));
+        return m;
+    }
+}
+
+// Position of the k-th lowest set bit (k >= 1) of a mask that holds at least k.
+__device__ __forceinline__ int nth_bit(uint32_t m, int k) {
+    int pos = 0;
+    int c = __popc(m & 0xffffu);
+    if (k > c) {
+        k -= c;
+        m >>= 16;
+        pos = 16;
+    }
+    c = __popc(m & 0xffu);
+    if (k > c) {
+        k -= c;
+        m >>= 8;
+        pos += 8;
+    }
+    for (; k > 1; --k) m &= m - 1;
+    return pos + 31 - __clz(m & (0u - m));
+}
+
+// Exact selection by ballot scans of the omnigram (Sec. 4.1, Sec. 4.2), one window for the whole
+// warp, 32 entries a step. Given a pivot rank p and c = #{window members with rank < p}, returns the
+// rank m of the window element with window-rank `target`. All 32 lanes pass the same arguments and
+// get the same result; -1 means the counts were inconsistent (never expected). (Two or four
+// entries per lane and step take fewer steps but more population counts, whose rate is an eighth
+// of an addition's: the seed rows' phase 31k -> 36k and 47k cycles per u16 r = 48 tile.)
+template <int SHAPE, int W>
+__device__ __forceinline__ int warp_select(const typename Loc<W>::E* __restrict__ om, int N, int p, int c,
+                                           int target, int px, int py, const Member<SHAPE, W>& member) {
     const int lane = threadIdx.x & 31;
+    WordTest<SHAPE, W> wt;
+    wt.init(member, px, py);
     if (c <= target) {  // the answer is at or above p
         int need = target - c + 1;
         for (int v0 = p; v0 < N; v0 += 32) {
             const int v = v0 + lane;
-            const bool in = v < N && member(om[v], px, py);
+            const bool in = v < N && wt.lo(om[v]) < 0;
             const uint32_t mask = __ballot_sync(kFull, in);
             const int cnt = __popc(mask);
             if (cnt >= need) {
                 const uint32_t hit = __ballot_sync(kFull, in && __popc(mask & lanemask_le()) == need);
-                return v0 + __ffs(hit) - 1;
+                return v0 + 31 - __clz(hit);
             }
             need -= cnt;
         }
@@ -252,12 +344,12 @@ __device__ __forceinline__ int ballot_select(const E* __restrict__ om, int N, in
         int need = c - target;
         for (int v1 = p; v1 > 0; v1 -= 32) {
             const int v = v1 - 32 + lane;
-            const bool in = v >= 0 && member(om[v], px, py);
+            const bool in = v >= 0 && wt.lo(om[v]) < 0;
             const uint32_t mask = __ballot_sync(kFull, in);
             const int cnt = __popc(mask);
             if (cnt >= need) {
                 const uint32_t hit = __ballot_sync(kFull, in && __popc(mask & lanemask_ge()) == need);
-                return v1 - 32 + __ffs(hit) - 1;
+                return v1 - 1 - __clz(hit);
             }
             need -= cnt;
         }
@@ -266,7 +358,7 @@ __device__ __forceinline__ int ballot_select(const E* __restrict__ om, int N, in
 }
 
 // Warp-cooperative exact selection for long walks (seed windows): the same contract as
-// ballot_select, but every lane tests two consecutive aligned 128-bit groups of entries per
+// warp_select, but every lane tests two consecutive aligned 128-bit groups of entries per
 // step, so a warp covers 64 groups (512 entries of 16 bits) per step. A warp reduction of the
 // per-lane member counts says whether the step holds the target; only that last step takes the
 // warp prefix sum that finds the lane, and the lane picks the entry. Entries past N up to the
@@ -370,108 +462,164 @@ __device__ __forceinline__ int window_rows_below(const int* spans, int nrows, co
 }
 
 // Per-thread exact selection (vertical sweep): every lane refines its own window. It scans the
-// omnigram from its pivot in aligned groups of entries (one 128-bit load), K groups per step
-// (the loop's votes and bookkeeping are paid once per K groups: K = 4 where scans are short,
-// small kernels; 8 where they are long), counting members, until the group holding the
-// target-th member. While at least kHandoff lanes are still
-// scanning this is the cheapest schedule; the last few lanes of a warp (long jumps at edges and
-// impulses) are finished by warp-cooperative ballot scans instead of keeping 29+ lanes idle.
-// Same contract as ballot_select, per lane. All loops are bounded by the omnigram length.
-constexpr int kHandoff = 8;
-constexpr int kHandoffAfterGroups = 8;
+// omnigram from its pivot in aligned 64-byte blocks, builds each block's membership mask, and
+// stops at the block that holds the target-th member. A warp repeats the block step until its
+// longest scan is done; only a few lanes left after many blocks (jumps at edges and impulses) are
+// finished one at a time by warp-wide scans.
+// Bound by instruction issue: a block takes 64 dot products, 32 masks and 32 shifts, which share
+// the issue slots of two half-rate pipes (u16 r = 48: 6.7 blocks per warp and step, 35 % of the
+// kernel's instructions). Against scans of 4 or 8 unaligned groups per step with compares and a
+// hand-off after 8 groups, the vertical sweep of a u16 r = 48 tile went from 237k to 169k cycles
+// together with the packed slide below; a hand-off as early as that costs five warp-wide scans
+// per step.
+// Arguments: pivot p, members below it c, target t; returns m (-1: inconsistent). Sentinels fill
+// the omnigram's last block. All loops are bounded by the omnigram length.
+constexpr int kHandoff = 3;
+constexpr int kHandoffAfterBlocks = 16;
 
-// KS > 0: KS groups per step, fixed at compile time; KS = 0: `groups` per step (at most 8),
-// read at run time (smaller code).
-template <int SHAPE, int W, int KS>
-__device__ __forceinline__ int thread_select(const typename Loc<W>::E* __restrict__ om, int N, int p, int c,
-                                             int target, int px, int py, const Member<SHAPE, W>& member,
-                                             int groups = KS) {
-    constexpr int kUnroll = KS > 0 ? KS : 8;
-    const int K = KS > 0 ? KS : groups;
-    const int handoff_after = (kHandoffAfterGroups + K - 1) / K;  // steps
-    constexpr int G = Loc<W>::kGroup;
-    constexpr uint32_t kAll = (1u << G) - 1;
-    const int lane = threadIdx.x & 31;
+template <int SHAPE, int W>
+__device__ __forceinline__ int lane_select(const typename Loc<W>::E* __restrict__ om, int N, int p, int c, int t,
+                                           int px, int py, const Member<SHAPE, W>& member) {
+    constexpr int kBlockShift = W == 0 ? 5 : 4;
+    constexpr int kBlock = 1 << kBlockShift;  // entries per block
+    constexpr uint32_t kAll = kBlock == 32 ? 0xffffffffu : (1u << kBlock) - 1;
+    const uint4* om128 = reinterpret_cast<const uint4*>(om);
+    const int blast = (N - 1) >> kBlockShift;
+    const bool up = c <= t;
+    int need = up ? t - c + 1 : c - t;
+    const int v = up ? p : max(p - 1, 0);  // next entry to examine
+    int b = v >> kBlockShift;
+    // the pivot's block counts on the pivot's side only
+    uint32_t first = up ? kAll << (v & (kBlock - 1)) : kAll >> (kBlock - 1 - (v & (kBlock - 1)));
     WordTest<SHAPE, W> wt;
     wt.init(member, px, py);
-    const uint4* om128 = reinterpret_cast<const uint4*>(om);
-    const bool up = c <= target;
-    int need = up ? target - c + 1 : c - target;
-    int nextv = up ? p : p - 1;  // next omnigram entry to examine
-    const int glast = (N - 1) / G;
-    bool done = false;
-    int m = -1;
-    // Entries past N up to the last group's end are sentinels that are never members, so only
-    // the first group needs a mask: the entries on the far side of the pivot.
-    const int o0 = nextv & (G - 1);
-    uint32_t first = up ? (kAll << o0) & kAll : kAll >> (G - 1 - o0);
-    constexpr int kShift = G == 8 ? 3 : 2;
-    for (int it = 0; it <= glast + 1; ++it) {
-        // the hand-off test costs a vote, so it only starts once the typical scan is over
-        if (it >= handoff_after && __popc(__ballot_sync(kFull, !done)) < kHandoff) break;
-        if (it < handoff_after && !__any_sync(kFull, !done)) break;
-        if (!done) {
-            const int g = nextv >> kShift;  // -1 below entry 0
-            if ((unsigned)g > (unsigned)glast) {
-                done = true;
-            } else {
-                constexpr int kb = G / 4;  // entries per word
-                uint32_t selmask = 0;
-                int selg = 0;
-                bool found = false;
-#pragma unroll
-                for (int k = 0; k < kUnroll; ++k) {
-                    if (KS == 0 && k >= K) break;  // uniform: every lane has the same K
-                    const int gk = up ? g + k : g - k;
-                    const bool ok = (unsigned)gk <= (unsigned)glast;
-                    const uint4 q = om128[ok ? gk : g];
-                    uint32_t mk = wt(q.x) | (wt(q.y) << kb) | (wt(q.z) << (2 * kb)) | (wt(q.w) << (3 * kb));
-                    if (!ok) mk = 0;
-                    if (k == 0) mk &= first;
-                    const int c = __popc(mk);
-                    if (!found) {
-                        if (c >= need) {
-                            found = true;
-                            selmask = mk;
-                            selg = gk;
-                        } else {
-                            need -= c;
-                        }
-                    }
-                }
-                first = kAll;
-                if (found) {
-                    uint32_t mask = selmask;
-                    if (up) {
-                        for (int k = 1; k < need; ++k) mask &= mask - 1;  // drop the lowest need-1
-                        m = G * selg + __ffs(mask) - 1;
-                    } else {
-                        for (int k = 1; k < need; ++k) mask ^= 1u << (31 - __clz(mask));  // drop the highest
-                        m = G * selg + 31 - __clz(mask);
-                    }
-                    done = true;
-                } else {
-                    nextv = up ? G * (g + K) : G * (g - K + 1) - 1;
-                }
+    uint32_t mask = 0;  // the block that holds the answer: its members, their number, and its place in b
+    int cnt = 0;
+    bool todo = true;
+    for (int it = 0; it <= blast + 1; ++it) {
+        const uint32_t alive = __ballot_sync(kFull, todo);
+        if (alive == 0) break;
+        if (it >= kHandoffAfterBlocks && __popc(alive) < kHandoff) break;
+        if (todo) {
+            mask = block_mask<SHAPE, W>(om128, b, wt) & first;
+            cnt = __popc(mask);
+            first = kAll;
+            todo = cnt < need;
+            if (todo) {
+                need -= cnt;
+                b += up ? 1 : -1;
+                if ((unsigned)b > (unsigned)blast) todo = false, mask = 0;  // ran off the omnigram
             }
         }
     }
-    // hand-off: the remaining lanes, one window at a time, by ballot scans
-    uint32_t rest = __ballot_sync(kFull, !done);
+    int m = -1;
+    if (!todo && mask != 0) m = kBlock * b + nth_bit(mask, up ? need : cnt - need + 1);
+    uint32_t rest = __ballot_sync(kFull, todo);
     while (rest) {
         const int j = __ffs(rest) - 1;
         rest &= rest - 1;
         const int upj = __shfl_sync(kFull, (int)up, j);
-        const int nj = __shfl_sync(kFull, nextv, j);
-        const int needj = __shfl_sync(kFull, need, j);
-        const int pxj = __shfl_sync(kFull, px, j);
-        const int pyj = __shfl_sync(kFull, py, j);
-        const int pj = upj ? nj : nj + 1;
-        const int cj = upj ? target + 1 - needj : target + needj;
-        const int mj = ballot_select(om, N, pj, cj, target, pxj, pyj, member);
-        if (lane == j) m = mj;
+        const int bj = __shfl_sync(kFull, b, j), nj = __shfl_sync(kFull, need, j);
+        const int pxj = __shfl_sync(kFull, px, j), pyj = __shfl_sync(kFull, py, j);
+        const int pj = upj ? kBlock * bj : kBlock * bj + kBlock;  // examined so far: all before (after) it
+        const int mj = warp_select<SHAPE, W>(om, N, pj, upj ? 0 : nj, upj ? nj - 1 : 0, pxj, pyj, member);
+        if ((int)(threadIdx.x & 31) == j) m = mj;
     }
     return m;
+}
+
+// ---- packed slides ---------------------------------------------------------------------------
+// Two windows one column apart read their ranks at any kernel column from the halves of one 32-bit
+// word of the ordinal image, if that word is aligned. PairBelow compares both halves with the
+// windows' pivots at once: with signed ranks (at most 32766) one add-min-relu instruction gives
+// [rank >= p] per half; ranks up to 65535 take two unsigned minima and a subtraction, giving
+// [rank < p]. `diff` adds the top entry's indicator minus the bottom entry's, so that a window
+// sliding down gains exactly the sum of diffs in members below its pivot (its bottom entries
+// enter, its top ones leave). The two halves accumulate in one word: differences may borrow across
+// the halves, and unpack_pair undoes it.
+template <bool S16>
+struct PairBelow {
+    uint32_t pv;  // S16: 1 - p per half, otherwise p per half
+    __device__ __forceinline__ void init(int p0, int p1) {
+        if constexpr (S16) {
+            p0 = 1 - p0;
+            p1 = 1 - p1;
+        }
+        pv = __byte_perm((uint32_t)p0, (uint32_t)p1, 0x5410);
+    }
+    __device__ __forceinline__ int diff(int acc, uint32_t top, uint32_t bot) const {
+        if constexpr (S16) {
+            return acc + (int)__viaddmin_s16x2_relu(top, pv, 0x00010001u) -
+                   (int)__viaddmin_s16x2_relu(bot, pv, 0x00010001u);
+        } else {
+            return acc + (int)__vminu2(pv - __vminu2(bot, pv), 0x00010001u) -
+                   (int)__vminu2(pv - __vminu2(top, pv), 0x00010001u);
+        }
+    }
+};
+
+__device__ __forceinline__ void unpack_pair(int acc, int* lo, int* hi) {
+    *lo = (int)(int16_t)(acc & 0xffff);
+    *hi = (acc - *lo) >> 16;
+}
+
+// Count change of every lane's window for one vertical step, lanes on adjacent columns. Each lane
+// takes the kernel columns whose words are aligned for its own window (box columns of its own
+// parity) and counts them for its window and the next lane's, so the warp reads and compares every
+// (window, column) pair once, two per instruction; each lane then adds the previous lane's high
+// half. The warp's first window has no previous lane: its other columns are split over the lanes.
+// `ctr` is the byte address of the window's centre in the ordinal image (one row above it for a
+// step up). `tab` lists the kernel columns as (top entry, bottom entry + 1) byte offsets, in units
+// of two columns of even box columns followed by two of odd ones; `units` such pairs. p is the
+// pivot as the ordinal image holds ranks. Returns the difference for a downward step.
+// Bound by issue: eight instructions (two loads, two compares, one accumulation, two addresses,
+// half a table load) per kernel column and two windows, against 18 for two 16-bit loads and
+// compares per window.
+template <bool S16, int kUnroll>
+__device__ __forceinline__ int slide(const unsigned char* ctr, const int4* tab, int units, int p) {
+    const int lane = threadIdx.x & 31;
+    const int pn = __shfl_down_sync(kFull, p, 1);
+    PairBelow<S16> pair;
+    pair.init(p, pn);
+    auto word = [](const unsigned char* q, int off) { return *reinterpret_cast<const uint32_t*>(q + off); };
+    const int4* mine = tab + (lane & 1);
+    int a = 0, a2 = 0;
+#pragma unroll kUnroll
+    for (int j = 0; j < units; ++j) {
+        const int4 o = mine[2 * j];
+        a = pair.diff(a, word(ctr, o.x), word(ctr, o.y));
+        a2 = pair.diff(a2, word(ctr, o.z), word(ctr, o.w));
+    }
+    // the first window's odd columns (its own column is even), one or two per lane
+    const unsigned char* c0 = ctr - 2 * lane;
+    const int pf = __shfl_sync(kFull, p, 0);
+    int s = 0;
+    for (int i = lane; i < 2 * units; i += 32) {
+        const int2 o = reinterpret_cast<const int2*>(tab + 1 + (i >> 1) * 2)[i & 1];
+        s += (int)(*reinterpret_cast<const uint16_t*>(c0 + o.y) < pf) -
+             (int)(*reinterpret_cast<const uint16_t*>(c0 + o.x) < pf);
+    }
+    s = __reduce_add_sync(kFull, s);
+    int lo, hi;
+    unpack_pair(a + a2, &lo, &hi);
+    const int prev = __shfl_up_sync(kFull, hi, 1);
+    return lo + (lane == 0 ? s : prev);
+}
+
+// Kernels of up to kScalarUnits units (12 columns) take slide_scalar: at 4096^2 u16 r = 4 it is 1.06x,
+// at u16 416x568 r = 5 1.11x the packed form, whose exchange costs about 80 instructions a step.
+constexpr int kScalarUnits = 3;
+// The same count change, every lane reading its own window's ranks one by one: for kernels of a few
+// columns, where the exchange between the lanes would cost more than it saves.
+__device__ __forceinline__ int slide_scalar(const unsigned char* ctr, const int4* tab, int units, int p) {
+    auto below = [&](int off) { return (int)(*reinterpret_cast<const uint16_t*>(ctr + off) < p); };
+    int d = 0;
+#pragma unroll 4
+    for (int j = 0; j < 2 * units; ++j) {
+        const int4 o = tab[j];
+        d += below(o.y) - below(o.x) + below(o.w) - below(o.z);
+    }
+    return d;
 }
 
 // Block-wide exclusive scan of 65536 16-bit counters packed two per word (bin 2k in the low
@@ -1165,6 +1313,14 @@ __device__ __forceinline__ T* place(unsigned char* smem, unsigned char* gslice, 
     return reinterpret_cast<T*>(loc >= 0 ? smem + loc : gslice + (-(long long)loc - 1));
 }
 
+// Fills the omnigram's last 64-byte block with sentinels no window contains.
+template <int W>
+__device__ __forceinline__ void pad_omnigram(typename Loc<W>::E* om, int N, int tid) {
+    constexpr int kBlock = 64 / (int)sizeof(typename Loc<W>::E);
+    const int pad = ((N + kBlock - 1) & ~(kBlock - 1)) - N;
+    if (tid < pad) om[N + tid] = Loc<W>::kSentinel;
+}
+
 // Several radii from one transform: keeps, in order, the omnigram entries that lie in a smaller
 // disk's footprint (`qfrow`: per box row, its columns lo | hi << 16; rows outside hold an empty
 // span), and gives those pixels their new ranks in the ordinal image. The order of the kept
@@ -1225,8 +1381,7 @@ __device__ int compact_omnigram(typename Loc<W>::E* om, int N, const int* qfrow,
         base += (int)wsum[32];
         G.sync();  // the offsets are read before the next chunk rewrites them
     }
-    const int pad = ((base + Loc<W>::kGroup - 1) & ~(Loc<W>::kGroup - 1)) - base;
-    if (tid < pad) om[base + tid] = Loc<W>::kSentinel;
+    pad_omnigram<W>(om, base, tid);
     G.sync();
     return base;
 }
@@ -1245,7 +1400,7 @@ template <int DT, int SHAPE, int W, int OG, int KS = 0, int XT = 0, int TMA = 1>
 __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned char* gslice, const Grp& G,
                                              TmaState* tma = nullptr, uint64_t* bar = nullptr,
                                              const void* tmap = nullptr) {
-    extern __shared__ __align__(16) unsigned char smem_base[];
+    extern __shared__ __align__(128) unsigned char smem_base[];
     unsigned char* const smem = smem_base + G.shift;  // this group's partition (tables excluded)
     using V = typename Traits<DT>::T;
     using E = typename Loc<W>::E;
@@ -1262,10 +1417,10 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
     const int cx0 = P.cx0, cy0 = P.cy0, xmin = P.xmin, ymin = P.ymin, hist_shift = P.hist_shift;
     // The ordinal image and the medians hold ranks minus rank_base, clamped to 16 bits: every
     // pivot lies in the tile's feasible median ranks (Fig. 10), which then compare exactly, so
-    // footprints beyond 65535 pixels keep a 16-bit ordinal image (rank_base = 0 below that).
-    const int rb = P.rank_base;
+    // footprints beyond 65535 pixels keep a 16-bit ordinal image and most others a signed one.
+    const int rb = P.rank_base, rel_max = P.rel_max;
 
-    const int2* vtab = reinterpret_cast<const int2*>(smem_base + P.off_vtab);
+    const int4* vtab = reinterpret_cast<const int4*>(smem_base + P.off_vtab);
     const int2* htab = reinterpret_cast<const int2*>(smem_base + P.off_htab);
     const int* spans = reinterpret_cast<const int*>(smem_base + P.off_spans);
     const int* frow = reinterpret_cast<const int*>(smem_base + P.off_frow);
@@ -1360,26 +1515,24 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
             for (int k = 0; k < 4; ++k) {
                 const int v = v0 + k * nthreads;
                 if (v < N)
-                    ord[(Loc<W>::y(e[k]) + cy0) * SP + Loc<W>::x(e[k]) + cx0] = (uint16_t)clampi(v - rb, 0, 65535);
+                    ord[(Loc<W>::y(e[k]) + cy0) * SP + Loc<W>::x(e[k]) + cx0] = (uint16_t)clampi(v - rb, 0, rel_max);
             }
         }
     } else {
         for (int v = tid; v < N; v += nthreads) {
             const uint32_t e = om[v];
-            ord[(Loc<W>::y(e) + cy0) * SP + Loc<W>::x(e) + cx0] = (uint16_t)clampi(v - rb, 0, 65535);
+            ord[(Loc<W>::y(e) + cy0) * SP + Loc<W>::x(e) + cx0] = (uint16_t)clampi(v - rb, 0, rel_max);
         }
     }
-    {   // pad the last 128-bit group with sentinels no window contains
-        const int pad = ((N + Loc<W>::kGroup - 1) & ~(Loc<W>::kGroup - 1)) - N;
-        if (tid < pad) om[N + tid] = Loc<W>::kSentinel;
-    }
+    pad_omnigram<W>(om, N, tid);
     G.sync();
 
     Member<SHAPE, W> member;
     if constexpr (SHAPE == kShapeDisk) {
         member.r2 = P.r2;
     } else {
-        member.spans = spans;
+        member.test = reinterpret_cast<const uint32_t*>(smem_base + P.off_test);
+        member.xmin = P.xmin;
         member.ymin = P.ymin;
         member.nrows = P.nrows;
     }
@@ -1394,24 +1547,23 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
     for (int q = 0; q < nr; ++q) {
         const int target = q == 0 ? P.rank : P.ranks[q];
         // the kernel of this target: the plan's own, or (several radii) the q-th disk's tables
-        const int2* qvtab = vtab;
+        const int4* qvtab = vtab;
         const int2* qhtab = htab;
         const int* qspans = spans;
-        int qn = P.n, qymin = ymin, qnrows = P.nrows, qncols = P.ncols;
+        int qn = P.n, qymin = ymin, qnrows = P.nrows, qunits = P.vunits;
         Member<SHAPE, W> qmember = member;
         if constexpr (XT == 1) {
             if (P.multi) {
-                qvtab = reinterpret_cast<const int2*>(smem_base + P.q_vtab[q]);
+                qvtab = reinterpret_cast<const int4*>(smem_base + P.q_vtab[q]);
                 qhtab = reinterpret_cast<const int2*>(smem_base + P.q_htab[q]);
                 qspans = reinterpret_cast<const int*>(smem_base + P.q_spans[q]);
                 qn = P.q_n[q];
                 qymin = P.q_ymin[q];
                 qnrows = P.q_nrows[q];
-                qncols = P.q_ncols[q];
+                qunits = P.q_vunits[q];
                 if constexpr (SHAPE == kShapeDisk) {
                     qmember.r2 = P.q_r2[q];
                 } else {
-                    qmember.spans = qspans;
                     qmember.ymin = qymin;
                     qmember.nrows = qnrows;
                 }
@@ -1511,7 +1663,7 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
                 const int below = window_rows_below(qspans, qnrows, ord + (cv + qymin) * SP + cu, SP, pivot - rb);
                 const int m = wide_select<SHAPE, W>(om, Nq, pivot, below, target, cu - cx0, cv - cy0, qmember);
                 if (m < 0) set_status(FIM_ERR_INTERNAL);
-                if (lane == 0) med[t * TX + s] = (uint16_t)(max(m, 0) - rb);
+                if (lane == 0) med[band * TX + s] = (uint16_t)(max(m, 0) - rb);
                 if (counting && lane == 0) {
                     const int kind = m < lo ? 2 : (m > hi ? 3 : 1);
                     atomicAdd(P.stats + 0, 1ull);
@@ -1538,7 +1690,9 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
                                 [&](int r) { atomicAdd(&hw[r >> qhist_shift], 1u); });
                     __syncwarp();
                     pivot = hist_pick(hw, 0, ts, &below) << qhist_shift;
-                    m = ballot_select(om, Nq, pivot, below, ts, cu - cx0, cv - cy0, qmember);
+                    // bin 0 also counts the members below the image's lowest rank
+                    if (pivot > 0) pivot += rb;
+                    m = warp_select<SHAPE, W>(om, Nq, pivot, below, ts, cu - cx0, cv - cy0, qmember);
                 } else {
                     if (P.seed_mode == kSeedWalk) {
                         // walk Omega from whichever end is known exactly: nothing lies below
@@ -1555,7 +1709,7 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
                     m = wide_select<SHAPE, W>(om, Nq, pivot, below, ts, cu - cx0, cv - cy0, qmember);
                 }
                 if (m < 0) set_status(FIM_ERR_INTERNAL);
-                if (lane == 0) med[t * TX + s] = (uint16_t)(max(m, 0) - rb);
+                if (lane == 0) med[band * TX + s] = (uint16_t)(max(m, 0) - rb);
                 if (sampling) {  // training row: features and the exact median's place in [lof, hif]
                     unsigned int row = 0;
                     if (lane == 0) row = atomicAdd(P.sample_count, 1u);
@@ -1586,7 +1740,7 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
             const int steps = right ? (GW - GW / 2 - 1) : (GW / 2);
             int cu = s - xmin;
             const int cv = t - ymin;
-            int p = med[t * TX + s] + rb;
+            int p = med[band * TX + s] + rb;
             constexpr int kRowsPerLane = (kMaxExtent + 31) / 32;
             int eo[kRowsPerLane], lo[kRowsPerLane];  // this lane's rows: entering / leaving offsets
     #pragma unroll
@@ -1612,10 +1766,10 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
                 cu += right ? 1 : -1;
                 s += right ? 1 : -1;
                 const int tn = mapped ? map_rank(P, tx0 + s, ty0 + t) : target;
-                const int m = ballot_select(om, Nq, p, tp + d, tn, cu - cx0, cv - cy0, qmember);
+                const int m = warp_select<SHAPE, W>(om, Nq, p, tp + d, tn, cu - cx0, cv - cy0, qmember);
                 if (m < 0) set_status(FIM_ERR_INTERNAL);
                 p = max(m, 0);
-                if (lane == 0) med[t * TX + s] = (uint16_t)(p - rb);
+                if (lane == 0) med[band * TX + s] = (uint16_t)(p - rb);
             }
         }
         G.sync();
@@ -1631,18 +1785,14 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
             const int groups = TX / 32;
             const int cg = warp % groups;
             const int rest = warp / groups;
-            const int vmix = XT == 1 && P.multi ? P.q_vmix[q] : P.vmix;
-            const int band = vmix ? (rest + lane) % P.RB : rest % P.RB;  // per lane with mixing
+            const int band = rest % P.RB;
             const int down = rest / P.RB;  // 0: up, 1: down
             const int s = cg * 32 + lane;
             int t = band * BH + BH / 2;
             const int steps = down ? (BH - BH / 2 - 1) : (BH / 2);
             const int cu = s - xmin;
             int cv = t - ymin;
-            int p = med[t * TX + s] + rb;
-            const int ncols = qncols;
-            const int scan_groups = P.scan_groups;
-            const int eoff = down ? 0 : -SP;
+            int p = med[band * TX + s] + rb;
             const Img im(P);
             char* const out = static_cast<char*>(q == 0 ? P.out : P.outs[q]);
             const int gx = tx0 + s;
@@ -1656,34 +1806,19 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
             };
             if (down) gather(p, t);  // the seed row's pixel
             for (int k = 0; k < steps; ++k) {
-                const uint16_t* ctr = ord + cv * SP + cu + eoff;
-                const int pr = p - rb;  // the pivot among the ordinal image's ranks
-                int d = 0;
-                // slide unrolled 8 kernel columns deep in the kernels compiled for the 1024-thread
-                // tiles (KS = 8), 4 in the others (measured, 4096^2 u16: r = 32-64 +1.2-1.8 % over
-                // 4; r = 2-16 -3 to -11 %; KS = 0 kernels serve small CTAs too)
-                constexpr int kSlideUnroll = KS == 8 ? 8 : 4;
-                if (down) {
-    #pragma unroll kSlideUnroll
-                    for (int j = 0; j < ncols; ++j) {
-                        const int2 o = qvtab[j];
-                        d += (int)(ctr[o.y] < pr) - (int)(ctr[o.x] < pr);
-                    }
-                } else {
-    #pragma unroll kSlideUnroll
-                    for (int j = 0; j < ncols; ++j) {
-                        const int2 o = qvtab[j];
-                        d += (int)(ctr[o.x] < pr) - (int)(ctr[o.y] < pr);
-                    }
-                }
+                const unsigned char* ctr = reinterpret_cast<const unsigned char*>(ord + (down ? cv : cv - 1) * SP + cu);
+                // slide unrolled deeper in the kernels of the 1024-thread tiles (KS = 8)
+                const int d = KS != 8 && qunits <= kScalarUnits ? slide_scalar(ctr, qvtab, qunits, p - rb)
+                              : P.s16 ? slide<true, KS == 8 ? 4 : 2>(ctr, qvtab, qunits, p - rb)
+                                      : slide<false, 2>(ctr, qvtab, qunits, p - rb);
                 const int tp = mapped ? map_rank(P, tx0 + s, ty0 + t) : target;
                 cv += down ? 1 : -1;
                 t += down ? 1 : -1;
                 const int tn = mapped ? map_rank(P, tx0 + s, ty0 + t) : target;
-                const int mine =
-                    thread_select<SHAPE, W, KS>(om, Nq, p, tp + d, tn, cu - cx0, cv - cy0, qmember, scan_groups);
-                if (mine < 0) set_status(FIM_ERR_INTERNAL);
-                p = max(mine, 0);
+                const int m =
+                    lane_select<SHAPE, W>(om, Nq, p, tp + (down ? d : -d), tn, cu - cx0, cv - cy0, qmember);
+                if (m < 0) set_status(FIM_ERR_INTERNAL);
+                p = max(m, 0);
                 if (pdst) *pdst = pval;  // the previous pixel's value has arrived by now
                 gather(p, t);
             }
@@ -1696,18 +1831,30 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
 }
 
 __device__ __forceinline__ void load_tables(const Plan& P) {
-    extern __shared__ __align__(16) unsigned char smem[];
+    extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, nt = blockDim.x;
     int2* vtab = reinterpret_cast<int2*>(smem + P.off_vtab);
+    const int nvtab = 4 * P.vunits;
     int2* htab = reinterpret_cast<int2*>(smem + P.off_htab);
     int* spans = reinterpret_cast<int*>(smem + P.off_spans);
     int* frow = reinterpret_cast<int*>(smem + P.off_frow);
-    for (int i = tid; i < P.ncols; i += nt) vtab[i] = make_int2(P.vtab[2 * i], P.vtab[2 * i + 1]);
+    for (int i = tid; i < nvtab; i += nt) vtab[i] = make_int2(P.vtab[2 * i], P.vtab[2 * i + 1]);
     for (int i = tid; i < P.nrows; i += nt) {
         htab[i] = make_int2(P.htab[2 * i], P.htab[2 * i + 1]);
         spans[i] = P.spans[i];
     }
     for (int i = tid; i < P.SH; i += nt) frow[i] = P.frow[i];
+    if (P.off_test >= 0) {  // the span test's words, kSpanCopies of each row and of the empty one
+        uint32_t* test = reinterpret_cast<uint32_t*>(smem + P.off_test);
+        for (int i = tid; i < (P.nrows + 1) * kSpanCopies; i += nt) {
+            const int r = i / kSpanCopies;
+            uint32_t t = 0x4000u << 16;
+            if (r < P.nrows)
+                t = (uint32_t)(0x8000 - (span_lo(P.spans[r]) - P.xmin + 256)) << 16 |
+                    (uint32_t)(0x7fff - (span_hi(P.spans[r]) - P.xmin + 256));
+            test[i] = t;
+        }
+    }
     if (P.xtab != nullptr) {
         int* xt = reinterpret_cast<int*>(smem + P.off_xtab);
         for (int i = tid; i < P.xtab_words; i += nt) xt[i] = P.xtab[i];
