@@ -367,6 +367,23 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
     // CTAs take 8-bit passes
     if (p->N > 65535 && p->sort != kSortCount8 && p->sort != kSortRadix16)
         p->sort = dtype == FIM_U16 && p->threads >= 1024 ? kSortCount16x2 : kSortRadix;
+    // Sort by equalised codes: float keys in full CTAs, footprints whose packed 16-bit places and
+    // 8-bit coordinates hold. About 1.5 codes per pixel, in units the scan splits evenly
+    // (layout_plan takes fewer where shared memory ends).
+    p->codes = 0;
+    if (p->sort == kSortRadix16 && p->N <= 65535 && !p->wide) {
+        const int unit = 256 * p->nwarps;
+        p->code_bits = 10;
+        p->codes = std::min(65536 / unit * unit - unit,
+                            (p->N + p->N / 2 + (1 << p->code_bits) + unit - 1) / unit * unit);
+        p->sample_step = 4;
+        p->nsample = 0;
+        for (int v = p->sample_step / 2; v < p->SH; v += p->sample_step)
+            p->nsample += (p->frow[v] >> 16) - span_lo_host(p->frow[v]) + 1;
+        p->nsample2 = 0;
+        for (int v = 0; v < p->SH; v += 2) p->nsample2 += (p->frow[v] >> 16) - span_lo_host(p->frow[v]) + 1;
+        if ((1 << p->code_bits) % p->threads != 0 || p->nsample == 0) p->codes = 0;
+    }
     // Placement. Tables, the ordinal image, medians and histograms always live in shared memory;
     // the omnigram, the radix keys and the radix position lists go to the CTA's global scratch
     // slice when shared memory cannot hold them (large kernels).
@@ -444,6 +461,7 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
     } else {
         const size_t keys_bytes = align16((size_t)p->S * p->SH * 4);
         const size_t dig_bytes = align16((size_t)p->S * p->SH);
+        const size_t tie_bytes = p->codes > 0 ? align16(((size_t)p->N / 32 + 2) * 4) : 0;
         const size_t hist_bytes = align16((size_t)p->nwarps * (kSortBins + 1) * 4);
         // try: (0) everything in shared memory; (1) keys in global; (2) keys and both lists in
         // global. Float keys in (1) and (2) keep list A in global memory too and give the stable
@@ -462,7 +480,7 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
                 if (mode < 2) need += om_bytes;  // B / omnigram
                 const size_t list_a = mode == 0 ? om_bytes : (use_dig ? dig_bytes : (mode == 1 ? om_bytes : 0));
                 const size_t sort_part = (mode == 0 ? keys_bytes : 0) + std::max(list_a + hist_bytes, bins_bytes);
-                need += std::max(sort_part, solve_bytes);
+                need += tie_bytes + std::max(sort_part, solve_bytes);
                 if (need <= (size_t)smem_limit) break;
             }
             if (mode < 3 || p->sort != kSortRadix16) break;
@@ -477,7 +495,15 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
             p->loc_b = take_glob(om_bytes);
         }
         p->loc_om = p->loc_b;  // the sorted positions are turned into the omnigram in place
+        p->loc_tie = (int)off;
+        off += tie_bytes;
         const size_t uni = off;
+        // the bins and tables of a sort by codes share the solve's region; as many codes as fit
+        p->loc_codes = (int)uni;
+        const size_t table_bytes = (size_t)12 << p->code_bits;
+        while (p->codes > 0 && uni + (size_t)p->codes * 2 + table_bytes > (size_t)smem_limit) p->codes -= 256 * p->nwarps;
+        if (p->codes < p->N / 2) p->codes = 0;
+        const size_t code_bytes = p->codes > 0 ? (size_t)p->codes * 2 + table_bytes : 0;
         if (mode == 0) {
             p->loc_keys = (int)off;
             off += keys_bytes;
@@ -502,7 +528,11 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
         p->loc_ord = (int)uni;
         p->loc_med = (int)(uni + ord_bytes);
         p->loc_shist = (int)(uni + ord_bytes + med_bytes);
-        smem = std::max(off, uni + solve_bytes);
+        smem = std::max(off, std::max(uni + solve_bytes, uni + code_bytes));
+        // The pixels' codes take the place of the radix sort's keys: in global scratch, or in shared
+        // memory past the bins (which, with the keys, bound what the radix sort needs there).
+        p->loc_cbuf = p->loc_keys < 0 ? p->loc_keys : (int)(uni + code_bytes);
+        if (p->loc_keys >= 0 && p->codes > 0) smem = std::max(smem, uni + code_bytes + align16((size_t)p->S * p->SH * 2));
     }
     if (smem > (size_t)smem_limit) return FIM_ERR_UNSUPPORTED;
     // Staging region for the footprint copies of interior tiles (128 bytes of slack let the kernel
@@ -1041,6 +1071,7 @@ fim_status fim_median_radii(const void* in, void* const* outs, const fim_kernel*
             p->outs[q] = outs[order[q]];
         }
         p->xtab_words = (int)xt.size();
+        p->codes = 0;  // the omnigram is narrowed from disk to disk: exact order
         s = layout_plan(p, smem_limit);
     }
     int* dx = nullptr;

@@ -18,6 +18,7 @@ constexpr int kMaxExtent = 264;   // kernel rows / columns held in a plan (>= FI
 constexpr int kMaxSide = 400;     // bounding-box rows of a tile footprint held in a plan
 constexpr int kSortBins = 256;    // 8-bit radix digits
 constexpr int kSeedBins = 256;    // coarse histogram bins of a seed solve
+constexpr int kMaxTie = 16;       // pixels of equal code (and different keys) a sort by codes leaves unordered
 constexpr int kSpanCopies = 8;    // copies of the span test's table, one per lane modulo 8
 constexpr int kMaxSignedRank = 32766;  // ordinal-image ranks the packed 16-bit compares take as signed
 
@@ -118,6 +119,10 @@ struct Plan {
     int hist_shift;         // seed histogram: bin = rank >> hist_shift
     int seed_mode;          // SeedMode of the plain seeds
     int sort;               // SortKind
+    int codes;              // sort by equalised codes: number of codes (0: `sort` alone)
+    int code_bits;          //   key bits of the first dealing table
+    int sample_step, nsample;  //   rows between the rows its first table is dealt by, pixels in them
+    int nsample2;           //   pixels of every second row (second table)
     int wide;               // 1: footprint box wider than 256: 32-bit omnigram entries and positions
     // learned rank bracket for the seed windows (all optional; null = the plain histogram seeds)
     const uint16_t* model;            // bf16 MLP parameters (kMlpParams), device memory
@@ -145,6 +150,7 @@ struct Plan {
     int groups;                                     // batches: tile groups of this job run per CTA
     int loc_om;                                     // omnigram (from the end of the sort on)
     int loc_bins;                                   // counting sorts: bins
+    int loc_codes, loc_tie, loc_cbuf;               // sort by codes: bins and tables; tie bits (kept); the codes
     int loc_keys, loc_a, loc_b, loc_hist;           // radix sort: keys, ping-pong lists, histograms
     int loc_dig;                                    // radix sort with keys in global scratch: digit bytes (-1: none)
     int loc_ord, loc_med, loc_shist;                // solve: ordinal image, seed rows' medians, seed histograms

@@ -263,10 +263,12 @@ fim_status run_filter(const void* in, void* out, int w, int h, size_t pitch, int
     // learned launches take the large-image shapes whatever the image size
     fim_status s = choose_tile(k, dtype, limit, &ts, 0, 0);
     if (s != FIM_OK) return s;
+    if (samples != nullptr && ts.Ty == 120) ts.Ty = 128;  // (120 rows only serve the scans)
     Plan* p = new (std::nothrow) Plan;
     if (!p) return FIM_ERR_OOM;
     s = make_plan(k, dtype, (k->n - 1) / 2, w, h, ts, limit, p);
     if (s == FIM_OK) {
+        p->codes = 0;  // the features are values at exact ranks
         p->in = in;
         p->out = out;
         p->pitch = (long long)pitch;

@@ -8,7 +8,9 @@
 //                          8-bit, and 16-bit data in 1024-thread CTAs: counting sort over 256 /
 //                                         65536 shared-memory bins, the bucket construction of
 //                                         Eq. 5 run by all threads;
-//                          float, and 16-bit data in smaller CTAs: LSD radix sort of
+//                          float in 1024-thread CTAs: counting sort by equalised 16-bit codes,
+//                                         ties settled at the output;
+//                          float otherwise, and 16-bit data in smaller CTAs: LSD radix sort of
 //                                         order-preserving keys (Sec. 4.1 float key), 8-bit
 //                                         passes (four / two).
 //   2. ordinal image   - I(Omega[v]) = v (Eq. 4), exact 16-bit ranks.
@@ -472,14 +474,14 @@ __device__ __forceinline__ int window_rows_below(const int* spans, int nrows, co
 // hand-off after 8 groups, the vertical sweep of a u16 r = 48 tile went from 237k to 169k cycles
 // together with the packed slide below; a hand-off as early as that costs five warp-wide scans
 // per step.
-// Arguments: pivot p, members below it c, target t; returns m (-1: inconsistent). Sentinels fill
-// the omnigram's last block. All loops are bounded by the omnigram length.
+// Arguments: pivot p, members below it c, target t; returns m (-1: inconsistent) and, in *members,
+// the members of m's block. Sentinels fill the omnigram's last block. All loops are bounded by the omnigram length.
 constexpr int kHandoff = 3;
 constexpr int kHandoffAfterBlocks = 16;
 
 template <int SHAPE, int W>
 __device__ __forceinline__ int lane_select(const typename Loc<W>::E* __restrict__ om, int N, int p, int c, int t,
-                                           int px, int py, const Member<SHAPE, W>& member) {
+                                           int px, int py, const Member<SHAPE, W>& member, uint32_t* members) {
     constexpr int kBlockShift = W == 0 ? 5 : 4;
     constexpr int kBlock = 1 << kBlockShift;  // entries per block
     constexpr uint32_t kAll = kBlock == 32 ? 0xffffffffu : (1u << kBlock) - 1;
@@ -501,7 +503,8 @@ __device__ __forceinline__ int lane_select(const typename Loc<W>::E* __restrict_
         if (alive == 0) break;
         if (it >= kHandoffAfterBlocks && __popc(alive) < kHandoff) break;
         if (todo) {
-            mask = block_mask<SHAPE, W>(om128, b, wt) & first;
+            *members = block_mask<SHAPE, W>(om128, b, wt);
+            mask = *members & first;
             cnt = __popc(mask);
             first = kAll;
             todo = cnt < need;
@@ -523,7 +526,10 @@ __device__ __forceinline__ int lane_select(const typename Loc<W>::E* __restrict_
         const int pxj = __shfl_sync(kFull, px, j), pyj = __shfl_sync(kFull, py, j);
         const int pj = upj ? kBlock * bj : kBlock * bj + kBlock;  // examined so far: all before (after) it
         const int mj = warp_select<SHAPE, W>(om, N, pj, upj ? 0 : nj, upj ? nj - 1 : 0, pxj, pyj, member);
-        if ((int)(threadIdx.x & 31) == j) m = mj;
+        if ((int)(threadIdx.x & 31) == j) {
+            m = mj;
+            if (m >= 0) *members = block_mask<SHAPE, W>(om128, m >> kBlockShift, wt);
+        }
     }
     return m;
 }
@@ -925,6 +931,289 @@ __device__ void ordinal_transform_count(const Plan& P, const int* frow, uint32_t
             }
         }
     }
+}
+
+// ---- ordinal transform by equalised codes --------------------------------------------------
+// Float keys have no counting sort of their own size, and an LSD radix sort's stable passes cost a
+// warp match per 32 pixels (64 cycles of the SM where the digits differ) and a scattered global
+// store. In full CTAs one counting sort places every pixel by a 16-bit code that follows the
+// tile's own distribution instead: histograms of a sample of the footprint over the keys' top bits
+// deal out codes in proportion, in two levels so that a tile whose values differ in their low
+// bits only is resolved as well, and within one bin the code is linear in the key. Codes never
+// decrease with the key, so pixels of different codes are in order; pixels of equal code (about
+// one other each) stay in any order, and `tie` has a bit per rank that shares its predecessor's
+// code. All counts, pivots and scans then work in this fixed total order, and the one place where
+// the order among equal codes matters, the value of a solved pixel, is settled there
+// (resolve_tie): for one pixel in five a comparison of two or three keys, instead of an exact order
+// of all the footprint's. (f32 8192^2 r = 64: the sort 227k -> 83k cycles per tile, the sweep
+// 143k -> 163k, the launch 13.2 -> 9.8 ms; the passes are bound by their shared-memory atomics
+// and table look-ups.)
+
+// Group of equal codes around rank v: its first rank, and one past its last. Rank 0 has no bit, and
+// a zero bit follows the last rank.
+__device__ __forceinline__ int tie_start(const uint32_t* tie, int v) {
+    int w = v >> 5;
+    uint32_t m = ~tie[w] & (0xffffffffu >> (31 - (v & 31)));
+    while (m == 0) m = ~tie[--w];
+    return 32 * w + 31 - __clz(m);
+}
+__device__ __forceinline__ int tie_end(const uint32_t* tie, int v) {
+    int w = (v + 1) >> 5;
+    uint32_t m = ~tie[w] & (0xffffffffu << ((v + 1) & 31));
+    while (m == 0) m = ~tie[++w];
+    return 32 * w + __ffs(m) - 1;
+}
+
+// The rank that holds the value of the window's element of rank m: where m shares its code with
+// other members of the window, the one with as many smaller members among them as precede m.
+// `mask` holds the members of m's 64-byte block, which a group rarely leaves; groups that do, and
+// groups with more than four members in the window, are walked entry by entry.
+template <class T, class K>
+__device__ __forceinline__ int resolve_tie(const uint16_t* om, const uint32_t* tie, int m, uint32_t mask, const T& wt,
+                                           K&& key_of) {
+    const uint32_t t = tie[m >> 5], next = tie[(m >> 5) + 1];
+    const uint32_t upto = 0xffffffffu >> (31 - (m & 31));  // entries of the block up to m
+    const uint32_t zlo = ~t & upto, zhi = ~t & ~upto;
+    if (zlo != 0 && (zhi != 0 || (next & 1u) == 0)) {  // the group lies in the block
+        // its entries: from the highest zero bit up to m on, below the lowest zero bit after m
+        const uint32_t group = (zhi != 0 ? (zhi & (0u - zhi)) - 1u : 0xffffffffu) & ~((1u << (31 - __clz(zlo))) - 1u);
+        uint32_t in = mask & group;
+        if ((in & (in - 1u)) == 0) return m;
+        const int before = __popc(in & (upto >> 1)), base = m & ~31;
+        const uint32_t low = in & (0u - in);
+        if (((in ^ low) & ((in ^ low) - 1u)) == 0) {  // two members
+            const int a = base + 31 - __clz(low), b = base + 31 - __clz(in);
+            const uint32_t ka = key_of(om[a]), kb = key_of(om[b]);
+            return (before == 0) == (ka <= kb) ? a : b;
+        }
+        int r[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {  // the members, in rank order; the last one repeats
+            r[i] = base + 31 - __clz(in & (0u - in));
+            const uint32_t rest = in & (in - 1u);
+            in = rest != 0 || i == 3 ? rest : in;
+        }
+        if (in == 0) {  // at most four
+            uint32_t k[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) k[i] = key_of(om[r[i]]);
+            int ans = m;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i > 0 && r[i] == r[i - 1]) continue;
+                int less = 0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (j != i && (j == 0 || r[j] != r[j - 1])) less += j < i ? k[j] <= k[i] : k[j] < k[i];
+                if (less == before) ans = r[i];
+            }
+            return ans;
+        }
+    }
+    const int s = tie_start(tie, m), e = tie_end(tie, m);
+    int n = 0, before = 0;
+    for (int u = s; u < e; ++u)
+        if (wt.lo(om[u]) < 0) {
+            ++n;
+            before += u < m;
+        }
+    if (n <= 1) return m;
+    // the members' distinct keys in ascending order, until one covers place `before`
+    uint32_t last = 0;
+    for (bool any = false;; any = true) {
+        uint32_t least = 0xffffffffu;
+        int at = -1, cnt = 0;
+        for (int u = s; u < e; ++u) {
+            if (wt.lo(om[u]) >= 0) continue;
+            const uint32_t k = key_of(om[u]);
+            if (any && k <= last) continue;
+            if (at < 0 || k < least) {
+                least = k;
+                at = u;
+                cnt = 0;
+            }
+            cnt += k == least;
+        }
+        if (at < 0 || before < cnt) return at < 0 ? m : at;
+        before -= cnt;
+        last = least;
+    }
+}
+
+// Deals out places in proportion to n counts (n a multiple of the group's threads): entry i becomes
+// its first place | its number of places << 16, one place plus floor(count * scale).
+__device__ void deal_places(uint32_t* t, int n, float scale, uint32_t* wtot, const Plan& P, const Grp& G) {
+    const int per = n / P.threads;
+    uint32_t sum = 0;
+    for (int j = 0; j < per; ++j) sum += 1u + (uint32_t)((float)t[G.tid * per + j] * scale);
+    uint32_t incl = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(kFull, incl, o);
+        if (G.lane >= o) incl += v;
+    }
+    if (G.lane == 31) wtot[G.warp] = incl;
+    G.sync();
+    uint32_t base = incl - sum;
+    for (int w = 0; w < G.warp; ++w) base += wtot[w];
+    for (int j = 0; j < per; ++j) {
+        const uint32_t c = 1u + (uint32_t)((float)t[G.tid * per + j] * scale);
+        t[G.tid * per + j] = base | (c << 16);
+        base += c;
+    }
+    G.sync();
+}
+
+// Exclusive scan of P.codes 16-bit counters packed two per word, as scan_bins16, setting the tie
+// bits of every code with more than one pixel. Returns the largest count this lane met.
+__device__ uint32_t scan_codes(uint32_t* bins, uint32_t* tie, uint32_t* wtot, const Plan& P, const Grp& G) {
+    const int lane = G.lane, warp = G.warp;
+    const int chunk = P.codes / 2 / P.nwarps;  // words per warp, a multiple of 128
+    uint4* b4 = reinterpret_cast<uint4*>(bins + warp * chunk);
+    uint32_t acc = 0;
+    for (int it = 0; it < chunk / 128; ++it) {
+        const uint4 q = b4[it * 32 + lane];
+        acc += ((q.x + (q.x >> 16)) & 0xffffu) + ((q.y + (q.y >> 16)) & 0xffffu) +
+               ((q.z + (q.z >> 16)) & 0xffffu) + ((q.w + (q.w >> 16)) & 0xffffu);
+    }
+    acc = __reduce_add_sync(kFull, acc);
+    if (lane == 0) wtot[warp] = acc;
+    G.sync();
+    uint32_t run = 0, most = 0;
+    for (int w = 0; w < warp; ++w) run += wtot[w];
+    for (int it = 0; it < chunk / 128; ++it) {
+        uint4 q = b4[it * 32 + lane];
+        const uint32_t s = ((q.x + (q.x >> 16)) & 0xffffu) + ((q.y + (q.y >> 16)) & 0xffffu) +
+                           ((q.z + (q.z >> 16)) & 0xffffu) + ((q.w + (q.w >> 16)) & 0xffffu);
+        uint32_t incl = s;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += t;
+        }
+        uint32_t b = run + incl - s;
+        uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t lo = w[k] & 0xffffu, hi = w[k] >> 16;
+            w[k] = b | ((b + lo) << 16);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t c = h ? hi : lo;
+                most = max(most, c);
+                uint32_t v = b + 1;  // ranks b + 1 .. b + c - 1 share their predecessor's code
+                b += c;
+                while (v < b) {
+                    const uint32_t len = min(b - v, 32u - (v & 31u));
+                    atomicOr(&tie[v >> 5], (0xffffffffu >> (32u - len)) << (v & 31u));
+                    v += len;
+                }
+            }
+        }
+        b4[it * 32 + lane] = make_uint4(w[0], w[1], w[2], w[3]);
+        run += __shfl_sync(kFull, incl, 31);
+    }
+    return most;
+}
+
+// Calls f(column, row, load(column, row)) for every footprint pixel of the rows v0, v0 + dv, ...: one
+// row per warp in turn, up to eight pixels of a lane loaded before the first call.
+template <class Ld, class Fn>
+__device__ __forceinline__ void each_pixel(const Plan& P, const int* frow, const Grp& G, int v0, int dv, Ld&& load,
+                                           Fn&& f) {
+    for (int v = v0 + G.warp * dv; v < P.SH; v += P.nwarps * dv) {
+        const int fr = frow[v], hi = span_hi(fr);
+        for (int u0 = span_lo(fr) + G.lane; u0 <= hi; u0 += 256) {
+            uint32_t x[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] = u0 + 32 * k <= hi ? load(u0 + 32 * k, v) : 0u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (u0 + 32 * k <= hi) f(u0 + 32 * k, v, x[k]);
+        }
+    }
+}
+
+// Builds the omnigram and the tie bits; false (to every thread) if the tile's groups of equal code
+// hold too many different keys, which then takes the radix sort. `work`: P.codes 16-bit bins,
+// then the dealing tables. `code` keeps every box position's code from the count to the scatter.
+template <int DT, int W, bool STAGED>
+__device__ bool ordinal_transform_codes(const Plan& P, const int* frow, uint32_t* work, uint32_t* tie, uint16_t* code,
+                                        uint32_t* misc, typename Loc<W>::E* om, const Footprint<DT>& fp, const Grp& G) {
+    const int tid = G.tid, N = P.N, nt = P.threads, nb = 1 << P.code_bits, shift = 32 - P.code_bits;
+    uint32_t* bins = work;
+    uint32_t* t1 = work + P.codes / 2;
+    uint32_t* t2 = t1 + nb;
+    const int nwords = P.codes / 2 + 3 * nb, ntie = N / 32 + 2;
+    for (int i = 4 * tid; i < nwords; i += 4 * nt) *reinterpret_cast<uint4*>(work + i) = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < ntie; i += nt) tie[i] = 0;
+    if (tid == 0) misc[36] = 0;
+    G.sync();
+    auto key = [&](int u, int v) { return fp.template key<STAGED>(u, v); };
+    // (scales rounded down: never more places than there are)
+    each_pixel(P, frow, G, P.sample_step / 2, P.sample_step, key,
+               [&](int, int, uint32_t k) { atomicAdd(&t1[k >> shift], 1u); });
+    G.sync();
+    deal_places(t1, nb, 0.9999f / (float)P.nsample * (float)nb, misc, P, G);
+    each_pixel(P, frow, G, 0, 2, key, [&](int, int, uint32_t k) {
+        const uint32_t e = t1[k >> shift];
+        atomicAdd(&t2[(e & 0xffffu) + __umulhi(k << P.code_bits, e >> 16)], 1u);
+    });
+    G.sync();
+    deal_places(t2, 2 * nb, 0.9999f / (float)P.nsample2 * (float)(P.codes - 2 * nb), misc, P, G);
+    auto code_of = [&](uint32_t k) -> uint32_t {
+        const uint32_t e = t1[k >> shift];
+        const unsigned long long p = (unsigned long long)(k << P.code_bits) * (e >> 16);
+        const uint32_t e2 = t2[(e & 0xffffu) + (uint32_t)(p >> 32)];
+        return (e2 & 0xffffu) + __umulhi((uint32_t)p, e2 >> 16);
+    };
+    each_pixel(P, frow, G, 0, 1, key, [&](int u, int v, uint32_t k) {
+        const uint32_t c = code_of(k);
+        code[v * P.S + u] = (uint16_t)c;
+        atomicAdd(&bins[c >> 1], 1u << ((c & 1u) << 4));
+    });
+    G.sync();
+    const uint32_t most = __reduce_max_sync(kFull, scan_codes(bins, tie, misc, P, G));
+    if (G.lane == 0) atomicMax(&misc[36], most);
+    G.sync();
+    each_pixel(P, frow, G, 0, 1, [&](int u, int v) -> uint32_t { return code[v * P.S + u]; },
+               [&](int u, int v, uint32_t c) {
+                   const uint32_t sh = (c & 1u) << 4;
+                   om[(atomicAdd(&bins[c >> 1], 1u << sh) >> sh) & 0xffffu] = Loc<W>::pack(u, v, P.cx0, P.cy0);
+               });
+    if (misc[36] <= (uint32_t)kMaxTie) return true;
+    // Some codes hold many pixels. Groups whose keys are all equal (impulses, flat areas, data of few
+    // distinct values) need no order: their tie bits go. A group with different keys keeps them.
+    G.sync();
+    uint32_t* mixed = work;          // bit s: the group that starts at rank s holds different keys
+    uint32_t* kept = work + ntie;
+    for (int i = tid; i < 2 * ntie; i += nt) work[i] = 0;
+    if (tid == 0) misc[36] = 0;
+    G.sync();
+    auto key_at = [&](int v) {
+        const uint32_t e = om[v];
+        return fp.template key<STAGED>(Loc<W>::x(e) + P.cx0, Loc<W>::y(e) + P.cy0);
+    };
+    for (int v = tid; v < N; v += nt)
+        if ((tie[v >> 5] >> (v & 31)) & 1u) {
+            const int s = tie_start(tie, v);
+            if (key_at(v) != key_at(s)) atomicOr(&mixed[s >> 5], 1u << (s & 31));
+        }
+    G.sync();
+    uint32_t largest = 0;
+    for (int v = tid; v < N; v += nt)
+        if ((tie[v >> 5] >> (v & 31)) & 1u) {
+            const int s = tie_start(tie, v);
+            if ((mixed[s >> 5] >> (s & 31)) & 1u) {
+                atomicOr(&kept[v >> 5], 1u << (v & 31));
+                largest = max(largest, (uint32_t)(v - s + 1));
+            }
+        }
+    largest = __reduce_max_sync(kFull, largest);
+    if (G.lane == 0) atomicMax(&misc[36], largest);
+    G.sync();
+    for (int i = tid; i < ntie; i += nt) tie[i] = kept[i];
+    const bool ok = misc[36] <= (uint32_t)kMaxTie;
+    G.sync();
+    return ok;
 }
 
 // LSD radix ordinal transform over bounding-box positions. Float keys in 1024-thread CTAs (C16):
@@ -1404,6 +1693,7 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
     unsigned char* const smem = smem_base + G.shift;  // this group's partition (tables excluded)
     using V = typename Traits<DT>::T;
     using E = typename Loc<W>::E;
+    constexpr bool kCodes = DT == FIM_F32 && W == 0 && KS != 4;  // plans may sort by codes
     const int tid = G.tid;
     const int lane = G.lane;
     const int warp = G.warp;
@@ -1431,6 +1721,7 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
     uint16_t* ord = reinterpret_cast<uint16_t*>(smem + P.loc_ord);
     uint16_t* med = reinterpret_cast<uint16_t*>(smem + P.loc_med);
     uint32_t* shist = reinterpret_cast<uint32_t*>(smem + P.loc_shist);
+    uint32_t* tie = reinterpret_cast<uint32_t*>(smem + P.loc_tie);
 
     // ---- 1. ordinal transform ------------------------------------------------------------------
     stamp(P, tile, 1, G);
@@ -1468,6 +1759,18 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
     // the sort, compiled for the staged box and for the image (one branch per tile)
     auto sort = [&](auto staged) {
         constexpr bool ST = decltype(staged)::value;
+        if constexpr (kCodes) {
+            if (P.codes > 0) {
+                // (a box that leaves the image repeats its edge pixels many times: exact order)
+                if (gx0 >= 0 && gy0 >= 0 && gx0 + P.S <= P.w && gy0 + P.SH <= P.h) {
+                    if (ordinal_transform_codes<DT, W, ST>(P, frow, reinterpret_cast<uint32_t*>(smem + P.loc_codes),
+                                                           tie, place<uint16_t>(smem, gslice, P.loc_cbuf), misc, om, fp, G))
+                        return;
+                    G.sync();
+                }
+                for (int i = tid; i < N / 32 + 2; i += nthreads) tie[i] = 0;
+            }
+        }
         if constexpr (DT == FIM_F32) {
             if (P.sort == kSortRadix16)
                 ordinal_transform_radix<DT, W, true, ST>(P, frow, place<uint32_t>(smem, gslice, P.loc_keys),
@@ -1798,13 +2101,33 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
             const int gx = tx0 + s;
             V pval = V(0);       // value gathered for the last solved pixel, not yet stored
             V* pdst = nullptr;   // where it goes (null: outside the image, or nothing pending)
-            auto gather = [&](int m, int tt) {
+            auto gather = [&](int m, int tt, uint32_t members) {
+                if constexpr (kCodes) {
+                    if (P.codes > 0) {  // (cv is the window's row)
+                        WordTest<SHAPE, W> wt;
+                        wt.init(qmember, cu - cx0, cv - cy0);
+                        // (only boxes inside the image have ties: no clamps)
+                        const char* mid = im.in + (long long)(gy0 + cy0) * im.pitch + (long long)(gx0 + cx0) * (int)sizeof(V);
+                        m = resolve_tie(om, tie, m, members, wt, [&](uint32_t e) {
+                            return Traits<DT>::key(__ldg(
+                                reinterpret_cast<const V*>(mid + (long long)Loc<W>::y(e) * im.pitch) + Loc<W>::x(e)));
+                        });
+                    }
+                }
                 const uint32_t e = om[m];
                 pval = load_px<DT>(im, gx0 + Loc<W>::x(e) + cx0, gy0 + Loc<W>::y(e) + cy0);
                 const int gy = ty0 + tt;
                 pdst = (gx < im.w && gy < im.h) ? reinterpret_cast<V*>(out + (long long)gy * im.pitch) + gx : nullptr;
             };
-            if (down) gather(p, t);  // the seed row's pixel
+            if (down) {  // the seed row's pixel
+                uint32_t members = 0;
+                if constexpr (kCodes) {
+                    WordTest<SHAPE, W> wt;
+                    wt.init(qmember, cu - cx0, cv - cy0);
+                    if (P.codes > 0) members = block_mask<SHAPE, W>(reinterpret_cast<const uint4*>(om), p >> 5, wt);
+                }
+                gather(p, t, members);
+            }
             for (int k = 0; k < steps; ++k) {
                 const unsigned char* ctr = reinterpret_cast<const unsigned char*>(ord + (down ? cv : cv - 1) * SP + cu);
                 // slide unrolled deeper in the kernels of the 1024-thread tiles (KS = 8)
@@ -1815,12 +2138,13 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
                 cv += down ? 1 : -1;
                 t += down ? 1 : -1;
                 const int tn = mapped ? map_rank(P, tx0 + s, ty0 + t) : target;
-                const int m =
-                    lane_select<SHAPE, W>(om, Nq, p, tp + (down ? d : -d), tn, cu - cx0, cv - cy0, qmember);
+                uint32_t members = 0;
+                const int m = lane_select<SHAPE, W>(om, Nq, p, tp + (down ? d : -d), tn, cu - cx0, cv - cy0, qmember,
+                                                    &members);
                 if (m < 0) set_status(FIM_ERR_INTERNAL);
                 p = max(m, 0);
                 if (pdst) *pdst = pval;  // the previous pixel's value has arrived by now
-                gather(p, t);
+                gather(p, t, members);
             }
             if (pdst) *pdst = pval;
         }
