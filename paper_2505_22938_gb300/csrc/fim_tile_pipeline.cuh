@@ -1064,8 +1064,10 @@ __device__ void deal_places(uint32_t* t, int n, float scale, uint32_t* wtot, con
 }
 
 // Exclusive scan of P.codes 16-bit counters packed two per word, as scan_bins16, setting the tie
-// bits of every code with more than one pixel. Returns the largest count this lane met.
-__device__ uint32_t scan_codes(uint32_t* bins, uint32_t* tie, uint32_t* wtot, const Plan& P, const Grp& G) {
+// bits of every code with 2 to kMaxTie pixels. Codes of more go to `list` (first rank | pixels << 16),
+// *listed of them.
+__device__ void scan_codes(uint32_t* bins, uint32_t* tie, uint32_t* list, uint32_t* listed, int cap, uint32_t* wtot,
+                           const Plan& P, const Grp& G) {
     const int lane = G.lane, warp = G.warp;
     const int chunk = P.codes / 2 / P.nwarps;  // words per warp, a multiple of 128
     uint4* b4 = reinterpret_cast<uint4*>(bins + warp * chunk);
@@ -1078,7 +1080,7 @@ __device__ uint32_t scan_codes(uint32_t* bins, uint32_t* tie, uint32_t* wtot, co
     acc = __reduce_add_sync(kFull, acc);
     if (lane == 0) wtot[warp] = acc;
     G.sync();
-    uint32_t run = 0, most = 0;
+    uint32_t run = 0;
     for (int w = 0; w < warp; ++w) run += wtot[w];
     for (int it = 0; it < chunk / 128; ++it) {
         uint4 q = b4[it * 32 + lane];
@@ -1098,7 +1100,12 @@ __device__ uint32_t scan_codes(uint32_t* bins, uint32_t* tie, uint32_t* wtot, co
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const uint32_t c = h ? hi : lo;
-                most = max(most, c);
+                if (c > (uint32_t)kMaxTie) {
+                    const uint32_t at = atomicAdd(listed, 1u);
+                    if (at < (uint32_t)cap) list[at] = b | (c << 16);
+                    b += c;
+                    continue;
+                }
                 uint32_t v = b + 1;  // ranks b + 1 .. b + c - 1 share their predecessor's code
                 b += c;
                 while (v < b) {
@@ -1111,7 +1118,6 @@ __device__ uint32_t scan_codes(uint32_t* bins, uint32_t* tie, uint32_t* wtot, co
         b4[it * 32 + lane] = make_uint4(w[0], w[1], w[2], w[3]);
         run += __shfl_sync(kFull, incl, 31);
     }
-    return most;
 }
 
 // Calls f(column, row, load(column, row)) for every footprint pixel of the rows v0, v0 + dv, ...: one
@@ -1145,7 +1151,7 @@ __device__ bool ordinal_transform_codes(const Plan& P, const int* frow, uint32_t
     const int nwords = P.codes / 2 + 3 * nb, ntie = N / 32 + 2;
     for (int i = 4 * tid; i < nwords; i += 4 * nt) *reinterpret_cast<uint4*>(work + i) = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < ntie; i += nt) tie[i] = 0;
-    if (tid == 0) misc[36] = 0;
+    if (tid == 0) misc[36] = misc[37] = 0;
     G.sync();
     auto key = [&](int u, int v) { return fp.template key<STAGED>(u, v); };
     // (scales rounded down: never more places than there are)
@@ -1171,49 +1177,38 @@ __device__ bool ordinal_transform_codes(const Plan& P, const int* frow, uint32_t
         atomicAdd(&bins[c >> 1], 1u << ((c & 1u) << 4));
     });
     G.sync();
-    const uint32_t most = __reduce_max_sync(kFull, scan_codes(bins, tie, misc, P, G));
-    if (G.lane == 0) atomicMax(&misc[36], most);
+    uint32_t* list = t1;  // (the codes are known: the tables are free)
+    const int cap = 3 * nb;
+    scan_codes(bins, tie, list, &misc[36], cap, misc, P, G);
     G.sync();
     each_pixel(P, frow, G, 0, 1, [&](int u, int v) -> uint32_t { return code[v * P.S + u]; },
                [&](int u, int v, uint32_t c) {
                    const uint32_t sh = (c & 1u) << 4;
                    om[(atomicAdd(&bins[c >> 1], 1u << sh) >> sh) & 0xffffu] = Loc<W>::pack(u, v, P.cx0, P.cy0);
                });
-    if (misc[36] <= (uint32_t)kMaxTie) return true;
-    // Some codes hold many pixels. Groups whose keys are all equal (impulses, flat areas, data of few
-    // distinct values) need no order: their tie bits go. A group with different keys keeps them.
-    G.sync();
-    uint32_t* mixed = work;          // bit s: the group that starts at rank s holds different keys
-    uint32_t* kept = work + ntie;
-    for (int i = tid; i < 2 * ntie; i += nt) work[i] = 0;
-    if (tid == 0) misc[36] = 0;
+    const int n = (int)misc[36];
+    if (n == 0) return true;
+    if (n > cap) return false;
+    // Codes of many pixels. Where all keys are equal (flat areas, impulses, data of few distinct values)
+    // the group needs no order; one with different keys leaves the tile to the radix sort. Groups of
+    // up to 1024 pixels take a warp each, larger ones the whole tile group.
     G.sync();
     auto key_at = [&](int v) {
         const uint32_t e = om[v];
         return fp.template key<STAGED>(Loc<W>::x(e) + P.cx0, Loc<W>::y(e) + P.cy0);
     };
-    for (int v = tid; v < N; v += nt)
-        if ((tie[v >> 5] >> (v & 31)) & 1u) {
-            const int s = tie_start(tie, v);
-            if (key_at(v) != key_at(s)) atomicOr(&mixed[s >> 5], 1u << (s & 31));
-        }
+    auto settle = [&](uint32_t first, uint32_t count, int from, int by) {
+        const uint32_t k0 = key_at((int)first);
+        bool same = true;
+        for (uint32_t i = 1 + from; i < count; i += by) same = same && key_at((int)(first + i)) == k0;
+        if (!same) misc[37] = 1;
+    };
+    for (int i = G.warp; i < n; i += P.nwarps)
+        if (list[i] >> 16 <= 1024u) settle(list[i] & 0xffffu, list[i] >> 16, G.lane, 32);
+    for (int i = 0; i < n; ++i)
+        if (list[i] >> 16 > 1024u) settle(list[i] & 0xffffu, list[i] >> 16, tid, nt);
     G.sync();
-    uint32_t largest = 0;
-    for (int v = tid; v < N; v += nt)
-        if ((tie[v >> 5] >> (v & 31)) & 1u) {
-            const int s = tie_start(tie, v);
-            if ((mixed[s >> 5] >> (s & 31)) & 1u) {
-                atomicOr(&kept[v >> 5], 1u << (v & 31));
-                largest = max(largest, (uint32_t)(v - s + 1));
-            }
-        }
-    largest = __reduce_max_sync(kFull, largest);
-    if (G.lane == 0) atomicMax(&misc[36], largest);
-    G.sync();
-    for (int i = tid; i < ntie; i += nt) tie[i] = kept[i];
-    const bool ok = misc[36] <= (uint32_t)kMaxTie;
-    G.sync();
-    return ok;
+    return misc[37] == 0;
 }
 
 // LSD radix ordinal transform over bounding-box positions. Float keys in 1024-thread CTAs (C16):
