@@ -263,7 +263,6 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
     p->G = ts.G;
     p->vthreads = 2 * ts.Tx * ts.RB;
     p->threads = std::max(p->vthreads, cta_threads);
-    p->scan_groups = p->threads < 1024 ? 4 : 8;
     p->nwarps = p->threads / 32;
     if (p->threads > 1024 || p->threads % 32 != 0) return FIM_ERR_UNSUPPORTED;  // 2 x Tx x bands threads
     p->shape = k->shape;
@@ -286,18 +285,26 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
     p->tiles_x = (w + ts.Tx - 1) / ts.Tx;
     p->tiles_y = (h + ts.Ty - 1) / ts.Ty;
     const int Tx = ts.Tx, Ty = ts.Ty, S = p->S, SP = p->SP;
-    // Footprint: the union of the kernel over the tile's output pixels, row by row (Fig. 10).
+    // Footprint: the union of the kernel over the tile's output pixels, row by row (Fig. 10): box row v
+    // meets kernel rows max(0, v - Ty + 1) .. min(nrows - 1, v). The least rlo and the greatest rhi of
+    // that moving range come from two queues of candidates (plans are tried for several tile heights
+    // on each call, and rescanning the range made a plan cost 30-50 us of host time).
     int64_t N = 0;
-    for (int v = 0; v < p->SH; ++v) {
-        const int i0 = std::max(0, v - Ty + 1), i1 = std::min(p->nrows - 1, v);
-        int lo = 1 << 30, hi = -(1 << 30);
-        for (int i = i0; i <= i1; ++i) {
-            lo = std::min(lo, k->rlo[i]);
-            hi = std::max(hi, k->rhi[i]);
+    {
+        int qlo[kMaxExtent], qhi[kMaxExtent], lo0 = 0, lo1 = 0, hi0 = 0, hi1 = 0;
+        for (int v = 0; v < p->SH; ++v) {
+            if (v < p->nrows) {
+                while (lo1 > lo0 && k->rlo[qlo[lo1 - 1]] >= k->rlo[v]) --lo1;
+                while (hi1 > hi0 && k->rhi[qhi[hi1 - 1]] <= k->rhi[v]) --hi1;
+                qlo[lo1++] = v;
+                qhi[hi1++] = v;
+            }
+            while (qlo[lo0] < v - Ty + 1) ++lo0;
+            while (qhi[hi0] < v - Ty + 1) ++hi0;
+            const int fl = k->rlo[qlo[lo0]] - k->xmin, fr = Tx - 1 + k->rhi[qhi[hi0]] - k->xmin;
+            p->frow[v] = (int)((uint32_t)(fl & 0xffff) | ((uint32_t)fr << 16));
+            N += fr - fl + 1;
         }
-        const int fl = lo - k->xmin, fr = Tx - 1 + hi - k->xmin;
-        p->frow[v] = (int)((uint32_t)(fl & 0xffff) | ((uint32_t)fr << 16));
-        N += fr - fl + 1;
     }
     // The ordinal image holds 16-bit ranks. Where the footprint has more than 32766 pixels they are
     // relative to the tile's feasible target ranks [rank, N - n + rank_hi] (Fig. 10), which is all
@@ -367,16 +374,19 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
     // CTAs take 8-bit passes
     if (p->N > 65535 && p->sort != kSortCount8 && p->sort != kSortRadix16)
         p->sort = dtype == FIM_U16 && p->threads >= 1024 ? kSortCount16x2 : kSortRadix;
-    // Sort by equalised codes: float keys in full CTAs, footprints whose packed 16-bit places and
-    // 8-bit coordinates hold. About 1.5 codes per pixel, in units the scan splits evenly
-    // (layout_plan takes fewer where shared memory ends).
+    // Sort by equalised codes: float keys in full CTAs, and float and 16-bit keys in CTAs of 256
+    // threads or more with enough pixels; footprints whose packed 16-bit places and 8-bit
+    // coordinates hold. About 1.5 codes per pixel, in units the scan splits evenly (layout_plan
+    // takes fewer where shared memory ends).
     p->codes = 0;
-    if (p->sort == kSortRadix16 && p->N <= 65535 && !p->wide) {
+    const bool lean = p->sort == kSortRadix && p->threads < 1024 && p->N >= 8000 && ts.Tx * ts.Ty >= 2048 &&
+                      p->threads >= (dtype == FIM_F32 ? 256 : 512);
+    if ((p->sort == kSortRadix16 || lean) && p->N <= 65535 && !p->wide) {
         const int unit = 256 * p->nwarps;
         p->code_bits = 10;
         p->codes = std::min(65536 / unit * unit - unit,
                             (p->N + p->N / 2 + (1 << p->code_bits) + unit - 1) / unit * unit);
-        p->sample_step = 4;
+        p->sample_step = dtype == FIM_F32 ? 4 : 2;
         p->nsample = 0;
         for (int v = p->sample_step / 2; v < p->SH; v += p->sample_step)
             p->nsample += (p->frow[v] >> 16) - span_lo_host(p->frow[v]) + 1;
@@ -471,20 +481,35 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
         // keeps the gathers. The 16-bit first pass's bins alias the region of list A (or the
         // digits) and the histograms, which are only used after it.
         const bool use_dig = p->dtype == FIM_F32;
+        // Plans of smaller CTAs that sort by codes take the radix sort for a few tiles only: its keys
+        // and list A stay in global scratch, so that the SM holds as many CTAs as its registers allow.
+        const bool lean = p->codes > 0 && p->sort == kSortRadix;  // (not changed by the fallback below)
+        const int share = device_smem_per_sm() / std::max(1, 65536 / (p->threads * 64)) / 128 * 128 - 1024;
         int mode = 0;
         for (;;) {
             const size_t bins_bytes = p->sort == kSortRadix16 ? 32768 * 4 : 0;
-            for (mode = 0; mode < 3; ++mode) {
+            for (mode = lean ? 1 : 0; mode < 3; ++mode) {
                 if (mode < 2 && p->wide) continue;  // 32-bit lists of a wide box never fit
                 size_t need = tab;
                 if (mode < 2) need += om_bytes;  // B / omnigram
-                const size_t list_a = mode == 0 ? om_bytes : (use_dig ? dig_bytes : (mode == 1 ? om_bytes : 0));
+                const size_t list_a = mode == 0 ? om_bytes : (use_dig ? dig_bytes : (mode == 1 && !lean ? om_bytes : 0));
                 const size_t sort_part = (mode == 0 ? keys_bytes : 0) + std::max(list_a + hist_bytes, bins_bytes);
                 need += tie_bytes + std::max(sort_part, solve_bytes);
                 if (need <= (size_t)smem_limit) break;
             }
-            if (mode < 3 || p->sort != kSortRadix16) break;
-            p->sort = kSortRadix;  // no room for the 65536 bins: four 8-bit passes
+            // No room for the 65536 bins, or only beside an omnigram in global scratch where the radix
+            // sort serves a few tiles (sort by codes): four 8-bit passes.
+            if (p->sort != kSortRadix16 || mode < 2 || (mode == 2 && (p->codes == 0 || p->wide))) break;
+            p->sort = kSortRadix;
+            if (mode == 2) {  // unless that spills as well
+                mode = 1;
+                const size_t need = tab + om_bytes + tie_bytes + std::max(dig_bytes + hist_bytes, solve_bytes);
+                if (need > (size_t)smem_limit) {
+                    p->sort = kSortRadix16;
+                    mode = 2;
+                }
+                break;
+            }
         }
         if (mode == 3) return FIM_ERR_UNSUPPORTED;
         size_t off = tab;
@@ -500,9 +525,17 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
         const size_t uni = off;
         // the bins and tables of a sort by codes share the solve's region; as many codes as fit
         p->loc_codes = (int)uni;
-        const size_t table_bytes = (size_t)12 << p->code_bits;
-        while (p->codes > 0 && uni + (size_t)p->codes * 2 + table_bytes > (size_t)smem_limit) p->codes -= 256 * p->nwarps;
-        if (p->codes < p->N / 2) p->codes = 0;
+        const size_t table_bytes = (size_t)(p->dtype == FIM_F32 ? 12 : 4) << p->code_bits;
+        if (p->codes > 0) {
+            const int unit = 256 * p->nwarps;
+            auto fitting = [&](size_t bytes) {
+                return bytes < uni + table_bytes ? 0 : (int)std::min<size_t>(p->codes, (bytes - uni - table_bytes) / 2 / unit * unit);
+            };
+            // a resident CTA less costs more than a few more pixels per code
+            const int shared = lean && uni + solve_bytes <= (size_t)share ? fitting((size_t)share) : 0;
+            p->codes = shared >= p->N - p->N / 4 ? shared : fitting((size_t)smem_limit);
+            if (p->codes < p->N / 2) p->codes = 0;
+        }
         const size_t code_bytes = p->codes > 0 ? (size_t)p->codes * 2 + table_bytes : 0;
         if (mode == 0) {
             p->loc_keys = (int)off;
@@ -510,7 +543,7 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
         } else {
             p->loc_keys = take_glob(keys_bytes);
         }
-        if (mode == 0 || (mode == 1 && !use_dig)) {
+        if (mode == 0 || (mode == 1 && !use_dig && !lean)) {
             p->loc_a = (int)off;
             off += om_bytes;
             p->loc_bins = p->loc_a;  // start of list A's and the histograms' region
@@ -561,6 +594,7 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
     }
     p->smem_bytes = (int)align16(smem);
     p->group_bytes = p->smem_bytes - p->tab_bytes;
+    p->scan_groups = p->threads < 1024 && p->codes == 0 ? 4 : 8;
     p->groups = 1;
     p->scratch_per_cta = (long long)glob;
     return FIM_OK;
@@ -614,10 +648,103 @@ static bool parse_tile_env(TileShape* ts) {
     return true;
 }
 
+fim_status default_tile(const fim_kernel* k, int dtype, int rank, int smem_limit, int w, int h, int cta_threads,
+                        bool exact_ranks, bool (*fits)(Plan&), Plan* p, TileShape* ts) {
+    const int extent = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1;
+    const int pw = w > 0 ? w : 1, ph = h > 0 ? h : 1;
+    auto valid = [&](const TileShape& c) {
+        return make_plan(k, dtype, rank, pw, ph, c, smem_limit, p, cta_threads, exact_ranks) == FIM_OK &&
+               p->smem_bytes <= smem_limit && (!fits || fits(*p));
+    };
+    // Waves of the image's tiles on the resident CTAs of the plan in *p (a batch or an unknown size
+    // counts as large).
+    auto waves = [&](const TileShape& c) {
+        if (w <= 0 || h <= 0) return 1e9;
+        return (double)((w + c.Tx - 1) / c.Tx) * ((h + c.Ty - 1) / c.Ty) / ((double)device_sm_count() * resident_ctas(*p));
+    };
+    // 1. Smaller CTAs, two or more to an SM, so that one's sort, seeds and barriers overlap another's
+    //    sweep. 8-bit data's 256 bins always allow it; float and 16-bit keys where the sort by codes
+    //    applies (16-bit data, whose counting sort is cheaper in a full CTA, gains least). Measured at
+    //    4096^2 against the one-CTA shapes: u8 r = 24 / 32 / 40 / 48 / 56 1.47x / 1.38x / 1.28x /
+    //    1.22x / 1.13x, f32 r = 16 / 20 / 24 / 32 / 40 / 48 1.13x / 1.25x / 1.21x / 1.11x / 1.08x /
+    //    1.04x, u16 r = 24 / 27 1.07x / 1.04x; u8 r = 64 and f32 r = 56, one CTA per SM, 1.0 and 0.9x.
+    //    An image of little over one wave of them has nothing to overlap.
+    struct Pref {
+        int dtype, lo, hi;  // kernel extents
+        TileShape ts;
+        int resident;  // CTAs per SM it must reach
+    };
+    static const Pref prefs[] = {{FIM_U8, 35, 67, {64, 40, 2, 2}, 3},  {FIM_U8, 68, 115, {64, 64, 4, 2}, 2},
+                                 {FIM_U8, 68, 115, {64, 48, 4, 2}, 2}, {FIM_U8, 68, 115, {64, 40, 4, 2}, 2},
+                                 {FIM_F32, 29, 34, {64, 64, 2, 2}, 3}, {FIM_F32, 35, 99, {64, 64, 4, 2}, 2},
+                                 {FIM_U16, 46, 59, {64, 64, 4, 2}, 2}};
+    for (const Pref& c : prefs)
+        if (c.dtype == dtype && c.lo <= extent && extent <= c.hi && valid(c.ts) && resident_ctas(*p) >= c.resident &&
+            (dtype == FIM_U8 || (p->codes > 0 && !exact_ranks)) && waves(c.ts) >= 1.25) {
+            *ts = c.ts;
+            return FIM_OK;
+        }
+    // 2. Small kernels: 32-column tiles in CTAs of 128 or 256 threads, many per SM (the footprint, and
+    //    so every scan, shrinks with the tile; 16-bit data then sorts by radix passes).
+    //    (u16 r = 18 / 22 32x64 1.04x / 1.07x over 32x32, both with four bands, on several waves.)
+    static const TileShape small[] = {{32, 32, 2, 1}, {32, 64, 4, 1}, {32, 32, 4, 1}};
+    if (extent <= 45)
+        for (int i = extent <= 33 ? 0 : 1; i < 3; ++i)
+            if (valid(small[i]) && (i != 1 || (dtype == FIM_U16 && waves(small[i]) >= 2.0))) {
+                *ts = small[i];
+                return FIM_OK;
+            }
+    // 3. 1024-thread CTAs, one to an SM, on 64-column tiles whose omnigram stays in shared memory: a
+    //    taller tile shares its sort and seeds among more rows, a lower one wastes less of the last
+    //    wave, whose tiles are not the average ones (own: a tile's fixed cost in rows; 16-bit
+    //    coordinates cost about 8 %;
+    //    u16 r = 72 / 88 64x96 / 64x48 1.10x / 1.39x over 64x64, f32 r = 72 1.14x, u8 r = 92 64x56
+    //    1.52x; f32 400x719 r = 51 64x48 2.3x over 64x128; in global scratch the omnigram's entries
+    //    cost each scan an L2 access).
+    static const int heights[] = {128, 112, 96, 88, 80, 72, 64, 56, 48, 40, 32};
+    auto cheapest = [&](double own, bool spilled, int least, bool coded) {
+        double best = 0.0;
+        for (int ty : heights) {
+            const TileShape c{64, ty, 8, 2};
+            if (ty < least || !valid(c) || (p->loc_om < 0) != spilled || (coded && p->codes == 0)) continue;
+            double cost = (ty + own) / ty * (p->wide ? 1.08 : 1.0);
+            if (w > 0 && h > 0) {
+                const double n = (double)((w + 63) / 64) * ((h + ty - 1) / ty) / device_sm_count();
+                cost *= std::max(ceil(n), n + 0.6) * ty;
+            }
+            if (best == 0.0 || cost < best) {
+                best = cost;
+                *ts = c;
+            }
+        }
+        return best > 0.0;
+    };
+    if (cheapest(0.27 * extent, false, w > 0 && h > 0 && (long long)w * h < 64LL * 48 * 304 ? 32 : 48, false)) return FIM_OK;
+    const TileShape low{64, 40, 4, 2};
+    if (dtype == FIM_U8 && valid(low) && p->loc_om >= 0) {  // (u8 r = 96: 1.31x over the spilled shapes)
+        *ts = low;
+        return FIM_OK;
+    }
+    // 4. The omnigram in global scratch: float tiles that still sort by codes (r = 96: 64x64 1.25x over
+    //    64x128), otherwise by cost, which for 8-bit and 16-bit data is nearly proportional to the
+    //    rows up to r = 96 (u16: 64x64 354k, 64x128 694k cycles) and less so above (r = 128: 64x64
+    //    587k, 64x88 696k), and for a float radix sort is not (r = 100: 64x128 1.2x over 64x64;
+    //    r = 128: 64x88 1.18x over 64x64): at least 88 rows where they fit.
+    if (dtype == FIM_F32 && (cheapest(3.0, true, 64, true) || cheapest(32.0, true, 88, false))) return FIM_OK;
+    if (cheapest(std::max(3.0, 0.9 * (extent - 193)), true, 64, false)) return FIM_OK;
+    static const TileShape last[] = {{32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
+    for (const TileShape& c : last)
+        if (valid(c)) {
+            *ts = c;
+            return FIM_OK;
+        }
+    return FIM_ERR_UNSUPPORTED;
+}
+
 fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape* ts, int w, int h,
-                       int cta_threads, bool exact_ranks) {
-    static const TileShape cands[] = {{32, 32, 2, 1}, {32, 32, 4, 1}, {64, 128, 8, 2}, {64, 120, 8, 2},
-                                      {64, 64, 8, 2}, {32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
+                       int cta_threads, bool exact_ranks, bool fixed_geometry) {
+    static const TileShape cands[] = {{32, 32, 2, 1}, {32, 32, 4, 1}, {64, 128, 8, 2}, {64, 64, 8, 2},
+                                      {32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
     TileShape forced;
     if (parse_tile_env(&forced)) {  // explicit override (experiments, tuning)
         Plan* p = new (std::nothrow) Plan;
@@ -643,24 +770,27 @@ fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape
             return FIM_OK;
         }
     }
-    // Defaults measured on the 4096^2 photo-like workload. Kernels up to 33 pixels across: 32x32
-    // tiles with two bands in 128-thread CTAs, many per SM (the footprint, and so every
-    // refinement scan, shrinks with the tile; 16-bit data then sorts by radix passes); up to 45
-    // across: the same tiles with four bands; up to 64 across: 64x64 tiles in 1024-thread CTAs;
-    // beyond: taller 64x128 tiles, which halve the seed and seed-row work per pixel.
+    if (!fixed_geometry) {
+        Plan* p = new (std::nothrow) Plan;
+        if (!p) return FIM_ERR_OOM;
+        // (small images are told by the tiles a large one takes)
+        fim_status s = default_tile(k, dtype, 0, smem_limit, 0, 0, cta_threads, exact_ranks, nullptr, p, ts);
+        TileShape small;
+        if (s == FIM_OK && w > 0 && h > 0) {
+            if (small_image_shape(k, dtype, w, h, smem_limit, cta_threads, exact_ranks, *ts, p, &small))
+                *ts = small;
+            else
+                s = default_tile(k, dtype, 0, smem_limit, w, h, cta_threads, exact_ranks, nullptr, p, ts);
+        }
+        delete p;
+        return s;
+    }
+    // Fixed geometry (training rows and the learned bracket, whose features and labels depend on the
+    // tile): kernels up to 33 pixels across 32x32 tiles with two bands, up to 45 across with four, up
+    // to 64 across 64x64, beyond 64x128; a shape of at least 64x64 that keeps the omnigram in shared
+    // memory before one that spills it; for 16-bit data the first exact-rank shape of at least 64x64.
     const int extent = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1;
-    const int first = extent <= 33 ? 0 : (extent <= 45 ? 1 : (extent >= 65 ? 2 : 4));
-    // Beyond the first valid shape, two measured exceptions (4096^2 photo-like u16, 4096^2 u8,
-    // 8192^2 f32):
-    // (1) where its omnigram spills to global scratch, a later shape of at least 64x64 whose
-    //     omnigram stays in shared memory wins (u16 r = 80: 5.04 Gpix/s on 64x64 against 3.37
-    //     on 64x128);
-    // (2) for 16-bit data, whose footprints beyond 65535 pixels (ranks relative to the feasible
-    //     range) count in two rounds and seed by walks, the first exact-rank shape wins unless
-    //     its tile is under 64x64 (r = 96: 3.01 on 64x64 against 2.82 on 64x128; r = 112: 2.31
-    //     on 64x128 against 0.88 on the exact-rank 32x64). 8-bit
-    //     data (256 bins) and float keys (radix passes on global lists at these sizes) keep the
-    //     larger tile (u8 r = 96: 4.30 on 64x128 against 3.43; f32 r = 100: 1.75 against 1.67).
+    const int first = extent <= 33 ? 0 : (extent <= 45 ? 1 : (extent >= 65 ? 2 : 3));
     struct Info {
         bool ok;
         int n;
@@ -701,15 +831,6 @@ fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape
             }
         }
     *ts = cands[pick];
-    // Small images, whose tiles would fill under half the GPU's resident CTAs: the first of the
-    // smaller shapes that fits them all in one wave (measured, u8 256^2 r = 4 / 16 / 32: 58 /
-    // 50 / 134 us per call on the default tiles against 23 / 26 / 33 on 32x8 tiles with 4 bands;
-    // 512^2: 63 / 63 / 160 against 36 / 40 / 54 on 32x16; at 1024^2 the defaults stay ahead).
-    Plan* p = new (std::nothrow) Plan;
-    if (!p) return FIM_ERR_OOM;
-    TileShape small;
-    if (small_image_shape(k, dtype, w, h, smem_limit, cta_threads, exact_ranks, *ts, p, &small)) *ts = small;
-    delete p;
     return FIM_OK;
 }
 

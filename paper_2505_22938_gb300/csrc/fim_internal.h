@@ -84,7 +84,7 @@ struct Plan {
     int Tx, Ty, txshift, RB, G;
     int threads, nwarps;    // CTA size (all cooperative loops and per-warp buffers)
     int vthreads;           // 2*Tx*RB: threads of the vertical sweep (the first ones of the CTA)
-    int scan_groups;        // kernel set: 8 the 1024-thread CTAs', 4 the smaller ones' (fim_tile_k4.cu)
+    int scan_groups;        // kernel set: 8 the 1024-thread CTAs' and the sort by codes, 4 the others (fim_tile_k4.cu)
     int S, SH;              // footprint bounding box (columns, rows)
     int SP;                 // row pitch (elements) of the ordinal image; SP/2 is odd
     int tiles_x, tiles_y;
@@ -227,7 +227,11 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
 fim_status plan_stage_model(Plan* p, int smem_limit);
 // Tile shape for an image of w x h (w or h <= 0: a batch, which fills the GPU like a large image).
 fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape* ts, int w, int h,
-                       int cta_threads = 0, bool exact_ranks = false);
+                       int cta_threads = 0, bool exact_ranks = false, bool fixed_geometry = false);
+// The untuned tile shape. `fits` (may be null) is one more condition on a candidate's plan; p is
+// storage for trial plans.
+fim_status default_tile(const fim_kernel* k, int dtype, int rank, int smem_limit, int w, int h, int cta_threads,
+                        bool exact_ranks, bool (*fits)(Plan&), Plan* p, TileShape* ts);
 int device_smem_limit();
 
 // Autotuner cache (fim_tune.cu).

@@ -6,8 +6,7 @@
 namespace fim {
 
 fim_status launch_tile_kernel_map(Plan& p, cudaStream_t stream) {
-    // one kernel set with the scan width read at run time keeps this unit quick to compile
-    return launch_tile_kernel_ks<0, 2>(p, stream);
+    return p.scan_groups == 8 ? launch_tile_kernel_ks<8, 2>(p, stream) : launch_tile_kernel_ks<0, 2>(p, stream);
 }
 
 fim_status read_and_clear_map_status() { return read_and_clear_unit_status(); }

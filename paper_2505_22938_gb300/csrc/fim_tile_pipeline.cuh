@@ -476,10 +476,18 @@ __device__ __forceinline__ int window_rows_below(const int* spans, int nrows, co
 // per step.
 // Arguments: pivot p, members below it c, target t; returns m (-1: inconsistent) and, in *members,
 // the members of m's block. Sentinels fill the omnigram's last block. All loops are bounded by the omnigram length.
-constexpr int kHandoff = 3;
-constexpr int kHandoffAfterBlocks = 16;
+// A block step costs about 165 instructions for any number of lanes, a hand-off 60 and 25 per 32
+// entries for one. In the small CTAs of small kernels, whose scans are one to three blocks, two
+// lanes are handed off after four blocks and up to four after eight (impulses: u16 4096^2 r = 4
+// 1181 -> 1097 us, 5th percentile r = 5 360 -> 338 us at 2048^2); with the long scans of large
+// kernels that costs 4-5 %, and only one or two lanes left after 16 blocks are.
+template <int KS>
+__device__ __forceinline__ bool hand_off(int blocks, uint32_t alive) {
+    if constexpr (KS == 8) return blocks >= 16 && __popc(alive) <= 2;
+    else return blocks >= 4 && __popc(alive) <= (blocks >= 8 ? 4 : 2);
+}
 
-template <int SHAPE, int W>
+template <int SHAPE, int W, int KS>
 __device__ __forceinline__ int lane_select(const typename Loc<W>::E* __restrict__ om, int N, int p, int c, int t,
                                            int px, int py, const Member<SHAPE, W>& member, uint32_t* members) {
     constexpr int kBlockShift = W == 0 ? 5 : 4;
@@ -501,7 +509,7 @@ __device__ __forceinline__ int lane_select(const typename Loc<W>::E* __restrict_
     for (int it = 0; it <= blast + 1; ++it) {
         const uint32_t alive = __ballot_sync(kFull, todo);
         if (alive == 0) break;
-        if (it >= kHandoffAfterBlocks && __popc(alive) < kHandoff) break;
+        if (hand_off<KS>(it, alive)) break;
         if (todo) {
             *members = block_mask<SHAPE, W>(om128, b, wt);
             mask = *members & first;
@@ -1148,25 +1156,31 @@ __device__ bool ordinal_transform_codes(const Plan& P, const int* frow, uint32_t
     uint32_t* bins = work;
     uint32_t* t1 = work + P.codes / 2;
     uint32_t* t2 = t1 + nb;
-    const int nwords = P.codes / 2 + 3 * nb, ntie = N / 32 + 2;
+    constexpr bool kTwo = DT == FIM_F32;              // 16-bit keys need one dealing level
+    constexpr int kKeyShift = DT == FIM_U16 ? 16 : 0;  // (the tables take 32-bit keys)
+    const int tables = kTwo ? 3 * nb : nb;
+    const int nwords = P.codes / 2 + tables, ntie = N / 32 + 2;
     for (int i = 4 * tid; i < nwords; i += 4 * nt) *reinterpret_cast<uint4*>(work + i) = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < ntie; i += nt) tie[i] = 0;
     if (tid == 0) misc[36] = misc[37] = 0;
     G.sync();
-    auto key = [&](int u, int v) { return fp.template key<STAGED>(u, v); };
+    auto key = [&](int u, int v) { return fp.template key<STAGED>(u, v) << kKeyShift; };
     // (scales rounded down: never more places than there are)
     each_pixel(P, frow, G, P.sample_step / 2, P.sample_step, key,
                [&](int, int, uint32_t k) { atomicAdd(&t1[k >> shift], 1u); });
     G.sync();
-    deal_places(t1, nb, 0.9999f / (float)P.nsample * (float)nb, misc, P, G);
+    deal_places(t1, nb, 0.9999f / (float)P.nsample * (float)(kTwo ? nb : P.codes - nb), misc, P, G);
+    if constexpr (kTwo) {
     each_pixel(P, frow, G, 0, 2, key, [&](int, int, uint32_t k) {
         const uint32_t e = t1[k >> shift];
         atomicAdd(&t2[(e & 0xffffu) + __umulhi(k << P.code_bits, e >> 16)], 1u);
     });
     G.sync();
     deal_places(t2, 2 * nb, 0.9999f / (float)P.nsample2 * (float)(P.codes - 2 * nb), misc, P, G);
+    }
     auto code_of = [&](uint32_t k) -> uint32_t {
         const uint32_t e = t1[k >> shift];
+        if constexpr (!kTwo) return (e & 0xffffu) + __umulhi(k << P.code_bits, e >> 16);
         const unsigned long long p = (unsigned long long)(k << P.code_bits) * (e >> 16);
         const uint32_t e2 = t2[(e & 0xffffu) + (uint32_t)(p >> 32)];
         return (e2 & 0xffffu) + __umulhi((uint32_t)p, e2 >> 16);
@@ -1178,7 +1192,7 @@ __device__ bool ordinal_transform_codes(const Plan& P, const int* frow, uint32_t
     });
     G.sync();
     uint32_t* list = t1;  // (the codes are known: the tables are free)
-    const int cap = 3 * nb;
+    const int cap = tables;
     scan_codes(bins, tie, list, &misc[36], cap, misc, P, G);
     G.sync();
     each_pixel(P, frow, G, 0, 1, [&](int u, int v) -> uint32_t { return code[v * P.S + u]; },
@@ -1688,7 +1702,10 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
     unsigned char* const smem = smem_base + G.shift;  // this group's partition (tables excluded)
     using V = typename Traits<DT>::T;
     using E = typename Loc<W>::E;
-    constexpr bool kCodes = DT == FIM_F32 && W == 0 && KS != 4;  // plans may sort by codes
+    // Plans that sort by codes run on these kernels only: the small CTAs of the others hold several
+    // phases in flight at once, and its code would crowd theirs out of the instruction cache (u16
+    // 4096^2 r = 16: 1289 -> 1392 us with it compiled in and not used).
+    constexpr bool kCodes = DT != FIM_U8 && W == 0 && KS == 8;
     const int tid = G.tid;
     const int lane = G.lane;
     const int warp = G.warp;
@@ -2134,7 +2151,7 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
                 t += down ? 1 : -1;
                 const int tn = mapped ? map_rank(P, tx0 + s, ty0 + t) : target;
                 uint32_t members = 0;
-                const int m = lane_select<SHAPE, W>(om, Nq, p, tp + (down ? d : -d), tn, cu - cx0, cv - cy0, qmember,
+                const int m = lane_select<SHAPE, W, KS>(om, Nq, p, tp + (down ? d : -d), tn, cu - cx0, cv - cy0, qmember,
                                                     &members);
                 if (m < 0) set_status(FIM_ERR_INTERNAL);
                 p = max(m, 0);

@@ -119,7 +119,7 @@ void tuned_clear() {
 // columns), tile height 16..128, 2..16 bands of at least 4 rows, 1..4 seeds per seed row.
 void tile_candidates(std::vector<TileShape>* out) {
     static const int txs[] = {64, 32};
-    static const int tys[] = {128, 64, 32, 16};
+    static const int tys[] = {128, 112, 96, 72, 64, 48, 40, 32, 16};
     static const int rbs[] = {2, 4, 8, 16};
     static const int gs[] = {1, 2, 4};
     for (int tx : txs)

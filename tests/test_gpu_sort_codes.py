@@ -1,5 +1,5 @@
-"""Parity of the sort by equalised codes (float) and of the radix sort (16-bit data in small CTAs)
-with the oracle, bit for bit (the output is a selected input value), on the value distributions
+"""Parity of the sort by equalised codes and of the radix sort (16-bit data in smaller CTAs) with
+the oracle, bit for bit (the output is a selected input value), on the value distributions
 that decide which pixels share a code: smooth data, values that differ in their last bits only,
 few distinct values, constants, impulses, both ends of the float order, and a mixture that must
 fall back to the exact sort. Sizes span several tiles of each shape with ragged edges.
@@ -41,7 +41,8 @@ def image(kind, dtype, h, w):
 
 
 @pytest.mark.parametrize("kind", ["photo", "constant", "narrow", "levels", "impulses", "ends", "mixed"])
-@pytest.mark.parametrize("r,tile", [(2, None), (8, "32,32,2,1"), (20, "64,64,8,2"), (33, "64,128,8,2")])
+@pytest.mark.parametrize("r,tile", [(2, None), (8, "32,32,2,1"), (20, "64,64,8,2"), (33, "64,128,8,2"),
+                                    (15, "64,64,2,2"), (24, "64,64,4,2")])
 def test_f32(kind, r, tile, monkeypatch):
     if tile:
         monkeypatch.setenv("FIM_TILE", tile)
@@ -51,9 +52,9 @@ def test_f32(kind, r, tile, monkeypatch):
 
 @pytest.mark.parametrize("kind", ["photo", "constant", "narrow", "levels", "impulses"])
 @pytest.mark.parametrize("spec,tile", [(("circle", 8), "32,32,2,1"), (("ellipse", 21, 9), "32,32,4,1"),
-                                       (("circle", 90), "32,64,4,1")])
+                                       (("circle", 90), "32,64,4,1"), (("circle", 24), "64,64,4,2")])
 @pytest.mark.parametrize("pct", [None, 0.0, 93.0])
-def test_u16_small_ctas(kind, spec, tile, pct, monkeypatch):
+def test_u16_smaller_ctas(kind, spec, tile, pct, monkeypatch):
     monkeypatch.setenv("FIM_TILE", tile)
     img = image(kind, "u16", 93, 107)
     off = oracle_offsets(*spec)
