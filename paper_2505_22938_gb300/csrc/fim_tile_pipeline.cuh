@@ -487,7 +487,7 @@ __device__ __forceinline__ bool hand_off(int blocks, uint32_t alive) {
     else return blocks >= 4 && __popc(alive) <= (blocks >= 8 ? 4 : 2);
 }
 
-template <int SHAPE, int W, int KS>
+template <int SHAPE, int W, int KS, bool kDense>
 __device__ __forceinline__ int lane_select(const typename Loc<W>::E* __restrict__ om, int N, int p, int c, int t,
                                            int px, int py, const Member<SHAPE, W>& member, uint32_t* members) {
     constexpr int kBlockShift = W == 0 ? 5 : 4;
@@ -503,28 +503,33 @@ __device__ __forceinline__ int lane_select(const typename Loc<W>::E* __restrict_
     uint32_t first = up ? kAll << (v & (kBlock - 1)) : kAll >> (kBlock - 1 - (v & (kBlock - 1)));
     WordTest<SHAPE, W> wt;
     wt.init(member, px, py);
-    uint32_t mask = 0;  // the block that holds the answer: its members, their number, and its place in b
+    // Large disks with the omnigram in shared memory (kDense): a lane that has found its block stays on
+    // it and computes the same mask again, so that the loop has no divergent branch (u16 r = 48 sweep
+    // 147k -> 140k cycles per tile). Where the idle lanes' loads cost more than the branch, they are
+    // masked off (hexagon R = 64 241k against 262k, u16 r = 128 221k against 262k, u16 r = 8 64k
+    // against 66k). Counts that do not add up end at the omnigram's first or last block and run into
+    // the limit.
+    const int dir = up ? 1 : -1;
+    uint32_t mask = 0;
     int cnt = 0;
     bool todo = true;
-    for (int it = 0; it <= blast + 1; ++it) {
-        const uint32_t alive = __ballot_sync(kFull, todo);
-        if (alive == 0) break;
-        if (hand_off<KS>(it, alive)) break;
-        if (todo) {
+    for (int it = 0;; ++it) {
+        if (kDense || todo) {
             *members = block_mask<SHAPE, W>(om128, b, wt);
             mask = *members & first;
             cnt = __popc(mask);
-            first = kAll;
             todo = cnt < need;
             if (todo) {
                 need -= cnt;
-                b += up ? 1 : -1;
-                if ((unsigned)b > (unsigned)blast) todo = false, mask = 0;  // ran off the omnigram
+                b = clampi(b + dir, 0, blast);
+                first = kAll;
             }
         }
+        const uint32_t alive = __ballot_sync(kFull, todo);
+        if (alive == 0 || it > blast || hand_off<KS>(it + 1, alive)) break;
     }
     int m = -1;
-    if (!todo && mask != 0) m = kBlock * b + nth_bit(mask, up ? need : cnt - need + 1);
+    if (!todo) m = kBlock * b + nth_bit(mask, up ? need : cnt - need + 1);
     uint32_t rest = __ballot_sync(kFull, todo);
     while (rest) {
         const int j = __ffs(rest) - 1;
@@ -1225,6 +1230,19 @@ __device__ bool ordinal_transform_codes(const Plan& P, const int* frow, uint32_t
     return misc[37] == 0;
 }
 
+// The valid lanes whose byte equals this lane's: eight votes (about 32 issue slots), where a warp match
+// takes two cycles of the SM per distinct value.
+__device__ __forceinline__ uint32_t same_byte(int d, bool valid) {
+    uint32_t peers = __ballot_sync(kFull, valid);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool bit = (d >> b) & 1;
+        const uint32_t m = __ballot_sync(kFull, bit);
+        peers &= bit ? m : ~m;
+    }
+    return peers;
+}
+
 // LSD radix ordinal transform over bounding-box positions. Float keys in 1024-thread CTAs (C16):
 // a 65536-bin counting pass on the low 16 bits (Eq. 5's construction, like 16-bit data) followed
 // by two stable 8-bit passes on the high bytes; otherwise 8-bit passes only, four for 32-bit
@@ -1237,7 +1255,7 @@ __device__ bool ordinal_transform_codes(const Plan& P, const int* frow, uint32_t
 // its digit of every box position into a shared byte array (`dig`, coalesced reads of the keys),
 // so that the passes look digits up in shared memory instead of gathering keys from L2 one by one.
 // The sorted positions end in list B, which is then rewritten in place as the omnigram.
-template <int DT, int W, bool C16, bool STAGED>
+template <int DT, int W, bool C16, bool STAGED, int KS>
 __device__ void ordinal_transform_radix(const Plan& P, const int* frow, uint32_t* keys, typename Loc<W>::Pos* bufA,
                                         typename Loc<W>::Pos* bufB, uint32_t* hist, uint32_t* wsum, uint32_t* bins,
                                         uint8_t* dig, const Footprint<DT>& fp, const Grp& G) {
@@ -1250,14 +1268,14 @@ __device__ void ordinal_transform_radix(const Plan& P, const int* frow, uint32_t
     // Exclusive scan of the per-warp digit counts in (digit, warp) order, in place: each thread
     // takes 8 consecutive counters (256 * nwarps counters over 32 * nwarps threads).
     auto scan_counts = [&]() {
-        const int e0 = tid * 8;
+        const int d0 = tid * 8 / nwarps, w0 = tid * 8 - d0 * nwarps;
         uint32_t c[8];
         uint32_t local = 0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int e = e0 + j, d = e / nwarps, wq = e - d * nwarps;
+        for (int j = 0, d = d0, wq = w0; j < 8; ++j) {
             c[j] = hist[wq * HS + d];
             local += c[j];
+            if (++wq == nwarps) wq = 0, ++d;
         }
         uint32_t incl = local;
         for (int o = 1; o < 32; o <<= 1) {
@@ -1278,10 +1296,10 @@ __device__ void ordinal_transform_radix(const Plan& P, const int* frow, uint32_t
         G.sync();
         uint32_t run = incl - local + wsum[warp];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int e = e0 + j, d = e / nwarps, wq = e - d * nwarps;
+        for (int j = 0, d = d0, wq = w0; j < 8; ++j) {
             hist[wq * HS + d] = run;
             run += c[j];
+            if (++wq == nwarps) wq = 0, ++d;
         }
     };
     // box position i lies in the footprint (Fig. 10)
@@ -1423,9 +1441,9 @@ __device__ void ordinal_transform_radix(const Plan& P, const int* frow, uint32_t
     const int seg = ((N + nwarps - 1) / nwarps + 31) & ~31;
     const int s0 = min(N, warp * seg), s1 = min(N, s0 + seg);
     // the stable passes, compiled for digits looked up in `dig` and for digits taken from the keys
-    auto stable_passes = [&](auto use_dig) {
-        constexpr bool kDig = decltype(use_dig)::value;
-        for (int pass = 0; pass < kPasses; ++pass) {
+    auto stable_pass = [&](auto use_dig, auto last, int pass) {
+        constexpr bool kDig = decltype(use_dig)::value, kLast = decltype(last)::value;
+        {
             const int shift = kBits0 + 8 * pass;
             if constexpr (kDig) {
                 const int nq = (area + 3) >> 2;  // keys of 4 consecutive box positions per load
@@ -1473,13 +1491,14 @@ __device__ void ordinal_transform_radix(const Plan& P, const int* frow, uint32_t
                 for (int k = 0; k < kG; ++k) {
                     if (b0 + 32 * k >= s1) break;
                     const bool valid = pos[k] >= 0;
-                    const uint32_t peers = __match_any_sync(kFull, d[k]);
+                    const uint32_t peers = kLast ? __match_any_sync(kFull, d[k]) : same_byte(d[k], valid);
                     uint32_t base = 0;
                     if (valid) base = hw[d[k]];
                     __syncwarp();
                     if (valid) {
-                        dst[base + __popc(peers & lanemask_lt())] = (Pos)pos[k];
-                        if (lane == __ffs(peers) - 1) hw[d[k]] = base + __popc(peers);
+                        const int earlier = __popc(peers & lanemask_lt());
+                        dst[base + earlier] = (Pos)pos[k];
+                        if (earlier == 0) hw[d[k]] = base + __popc(peers);
                     }
                     __syncwarp();
                 }
@@ -1488,6 +1507,15 @@ __device__ void ordinal_transform_radix(const Plan& P, const int* frow, uint32_t
             src = dst;
             dst = (dst == bufA) ? bufB : bufA;
         }
+    };
+    // A float key's top byte takes few values, which a match finds quickly; in the small CTAs the votes'
+    // code costs more instruction fetches than they save (f32 4096^2 r = 100 sort 543k -> 486k cycles
+    // per tile; u16 r = 8 1033 -> 1165 us with them).
+    constexpr int kSpread = KS != 8 ? 0 : (DT == FIM_F32 ? kPasses - 1 : kPasses);
+    auto stable_passes = [&](auto use_dig) {
+        for (int pass = 0; pass < kSpread; ++pass) stable_pass(use_dig, std::false_type{}, pass);
+        if constexpr (kSpread < kPasses)
+            for (int pass = kSpread; pass < kPasses; ++pass) stable_pass(use_dig, std::true_type{}, pass);
     };
     if constexpr (DT == FIM_F32) {  // only float plans place digits (one stable pass otherwise)
         if (dig != nullptr)
@@ -1785,21 +1813,21 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
         }
         if constexpr (DT == FIM_F32) {
             if (P.sort == kSortRadix16)
-                ordinal_transform_radix<DT, W, true, ST>(P, frow, place<uint32_t>(smem, gslice, P.loc_keys),
+                ordinal_transform_radix<DT, W, true, ST, KS>(P, frow, place<uint32_t>(smem, gslice, P.loc_keys),
                                                          place<typename Loc<W>::Pos>(smem, gslice, P.loc_a),
                                                          place<typename Loc<W>::Pos>(smem, gslice, P.loc_b),
                                                          reinterpret_cast<uint32_t*>(smem + P.loc_hist), misc,
                                                          reinterpret_cast<uint32_t*>(smem + P.loc_bins),
                                                          P.loc_dig >= 0 ? smem + P.loc_dig : nullptr, fp, G);
             else
-                ordinal_transform_radix<DT, W, false, ST>(P, frow, place<uint32_t>(smem, gslice, P.loc_keys),
+                ordinal_transform_radix<DT, W, false, ST, KS>(P, frow, place<uint32_t>(smem, gslice, P.loc_keys),
                                                           place<typename Loc<W>::Pos>(smem, gslice, P.loc_a),
                                                           place<typename Loc<W>::Pos>(smem, gslice, P.loc_b),
                                                           reinterpret_cast<uint32_t*>(smem + P.loc_hist), misc,
                                                           nullptr, P.loc_dig >= 0 ? smem + P.loc_dig : nullptr, fp,
                                                           G);
-        } else if (DT == FIM_U16 && P.sort == kSortRadix) {
-            ordinal_transform_radix<DT, W, false, ST>(P, frow, place<uint32_t>(smem, gslice, P.loc_keys),
+        } else if (DT == FIM_U16 && (KS == 4 || P.sort == kSortRadix)) {  // (fewer than 1024 threads: radix)
+            ordinal_transform_radix<DT, W, false, ST, KS>(P, frow, place<uint32_t>(smem, gslice, P.loc_keys),
                                                       place<typename Loc<W>::Pos>(smem, gslice, P.loc_a),
                                                       place<typename Loc<W>::Pos>(smem, gslice, P.loc_b),
                                                       reinterpret_cast<uint32_t*>(smem + P.loc_hist), misc, nullptr,
@@ -2151,7 +2179,7 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
                 t += down ? 1 : -1;
                 const int tn = mapped ? map_rank(P, tx0 + s, ty0 + t) : target;
                 uint32_t members = 0;
-                const int m = lane_select<SHAPE, W, KS>(om, Nq, p, tp + (down ? d : -d), tn, cu - cx0, cv - cy0, qmember,
+                const int m = lane_select<SHAPE, W, KS, SHAPE == kShapeDisk && OG == 0 && KS == 8>(om, Nq, p, tp + (down ? d : -d), tn, cu - cx0, cv - cy0, qmember,
                                                     &members);
                 if (m < 0) set_status(FIM_ERR_INTERNAL);
                 p = max(m, 0);
