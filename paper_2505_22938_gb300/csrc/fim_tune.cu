@@ -97,6 +97,7 @@ void save_locked() {
 bool tuned_lookup(const fim_kernel* k, int dtype, TileShape* ts, int size_cls, int cta_threads) {
     std::lock_guard<std::mutex> g(g_tune_mu);
     load_locked();
+    if (tune_map().empty()) return false;  // (every untuned call passes here: the device's name is slow to get)
     auto it = tune_map().find(Key(device_name(), dtype, kernel_hash(k), cta_threads, size_cls));
     if (it == tune_map().end()) return false;
     *ts = it->second;
