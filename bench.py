@@ -179,12 +179,13 @@ class ClockSampler:
 def algorithmic_ops_per_pixel(r: int, footprint: int, tile_w: int, tile_h: int, passes: int = 1,
                               width: int | None = None) -> float:
     """Element operations per output pixel: the ordinal transform touches every footprint
-    pixel once per sort pass (8-bit data and 16-bit data in 1024-thread CTAs: one counting-sort
-    pass; 16-bit data in smaller CTAs: two radix passes; float: three in 1024-thread CTAs, a 16-bit
-    counting pass and two 8-bit passes, else four), a vertical slide
-    compares the 2 * width entering and leaving pixels (width = 2r + 1 for a disk), and the
-    omnigram refinement tests at least one 64-entry block (the minimum when the median stays
-    within its pivot quantum). Each element operation needs at least one integer instruction."""
+    pixel once per sort pass (8-bit data, 16-bit data in 1024-thread CTAs and keys sorted by
+    equalised codes: one counting-sort pass; other 16-bit data: two radix passes; other float
+    data: three in 1024-thread CTAs, a 16-bit counting pass and two 8-bit passes, else four), a
+    vertical slide compares the 2 * width entering and leaving pixels (width = 2r + 1 for a disk),
+    and the omnigram refinement tests at least one 64-entry block (the minimum when the median
+    stays within its pivot quantum). Each element operation needs at least one integer
+    instruction."""
     w = 2 * r + 1 if width is None else width
     return footprint / (tile_w * tile_h) * passes + 2 * w + 64
 
@@ -193,10 +194,11 @@ def sort_passes(dtype: str, threads: int, footprint: int = 0) -> int:
     """Key passes of the ordinal transform the library runs for a plan (see the docstring above);
     footprints beyond 65535 pixels overflow the 16-bit counters of the 65536-bin pass: 16-bit
     data and the float keys' 16-bit pass count in two rounds of the same pass."""
-    if dtype == "f32":  # full CTAs: one 16-bit counting pass (two rounds beyond 65535) + two 8-bit passes
-        return 3 if threads >= 1024 else 4
+    coded = 8000 <= footprint <= 65535  # full CTAs, and smaller ones with enough pixels, sort by codes
+    if dtype == "f32":
+        return 1 if coded and threads >= 256 else (3 if threads >= 1024 else 4)
     if dtype == "u16" and threads < 1024:
-        return 2
+        return 1 if coded and threads >= 512 else 2
     if dtype == "u16" and footprint > 65535:  # the counting sort in two rounds over the key range
         return 2
     return 1

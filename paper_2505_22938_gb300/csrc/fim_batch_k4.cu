@@ -1,5 +1,4 @@
-// Batch class kernels with 4 omnigram groups per scan step (classes of the small-CTA tiles of
-// small kernels).
+// Batch class kernels of the kernel set for smaller CTAs.
 #include "fim_batch_launch.cuh"
 
 namespace fim {

@@ -1,4 +1,4 @@
-// Batch class kernels with 8 omnigram groups per scan step (classes of 1024-thread tiles).
+// Batch class kernels of the kernel set for 1024-thread CTAs and the sort by codes.
 #include "fim_batch_launch.cuh"
 
 namespace fim {

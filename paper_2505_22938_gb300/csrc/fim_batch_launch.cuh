@@ -1,11 +1,11 @@
 #pragma once
 // Batched persistent launch (device side): one persistent kernel per class of jobs that share a
-// tile-pipeline instantiation (dtype, kernel shape, omnigram encoding and home, scan width) and a
+// tile-pipeline instantiation (dtype, kernel shape, omnigram encoding and home, kernel set) and a
 // CTA size. A class kernel's CTAs take tiles from the class's device-side queue, which runs over
 // the tiles of all its jobs in the order the host sorted them (decreasing cost per tile), and
 // reload the plan of a tile's job when it changes. Each class kernel is the same specialised
 // pipeline as the single-image kernel of that class, at the CTA size its plans ask for. Included
-// by one translation unit per scan width, so that the two sets compile in parallel.
+// by one translation unit per kernel set, so that the two sets compile in parallel.
 #include "fim_tile_pipeline.cuh"
 
 namespace fim {

@@ -1,5 +1,5 @@
-// Single-image launches with 8 omnigram groups per scan step (the 1024-thread tiles of large
-// kernels) and the dispatch between the sets of kernels.
+// Single-image launches of the kernel set for 1024-thread CTAs and for smaller ones that sort by
+// codes, and the dispatch between the sets of kernels.
 #include "fim_tile_launch.cuh"
 
 namespace fim {

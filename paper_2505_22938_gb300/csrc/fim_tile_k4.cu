@@ -1,5 +1,5 @@
-// Single-image launches with 4 omnigram groups per scan step (the small-CTA tiles of small
-// kernels, where scans are short).
+// Single-image launches of the kernel set for smaller CTAs (the tiles of small kernels, and 8-bit
+// data's up to about 110 pixels across).
 #include "fim_tile_launch.cuh"
 
 namespace fim {

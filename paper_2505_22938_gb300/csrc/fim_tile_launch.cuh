@@ -1,6 +1,5 @@
 #pragma once
-// Single-image launches of the tile pipeline, for one number KS of omnigram groups per scan
-// step: each CTA takes Tx x Ty output tiles from a device-side queue and filters them one
+// Single-image launches of the tile pipeline, for one kernel set KS (see process_tile): each CTA takes Tx x Ty output tiles from a device-side queue and filters them one
 // after the other (Sec. 3.3, Sec. 4.2). Included by one translation unit per KS, so that the
 // two sets of kernels compile in parallel.
 #include <atomic>

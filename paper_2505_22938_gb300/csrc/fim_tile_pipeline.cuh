@@ -1712,8 +1712,10 @@ __device__ int compact_omnigram(typename Loc<W>::E* om, int N, const int* qfrow,
     return base;
 }
 
-// KS: omnigram groups per scan step of the vertical sweep, fixed at compile time (4 or 8; the
-// batch class kernels are compiled for both), or 0 to follow the plan's scan_groups at run time.
+// KS: the kernel set. 8: 1024-thread CTAs, and smaller ones that sort by codes (deeper unrolled
+// slides, scans without a divergent branch, the sort by codes); 4: the other, smaller CTAs, whose
+// several phases in flight share the instruction cache (short code); 0: extras and percentile maps
+// of those.
 // XT: 1 compiles the extras — the learned bracket, training-row output, seed statistics and
 // several target ranks per launch — and 2 a target rank per output pixel (a percentile map).
 // Each lives in kernels of its own: at the 64-register cap of 1024-thread CTAs their code
