@@ -116,15 +116,15 @@ fim_status fim_batch_create(const fim_job* jobs, int count, fim_batch** out) {
     if (limit <= 0) return FIM_ERR_CUDA;
     for (int i = 0; i < count; ++i) {
         const fim_job& j = jobs[i];
+        const int n = j.kernel->n;
+        PlanUse use{(n - 1) / 2};
+        if (j.percentile >= 0.0) use.rank = std::min(std::max((int)(j.percentile / 100.0 * (n - 1) + 0.5), 0), n - 1);
         TileShape ts;
         // a batch fills the GPU with the tiles of all its jobs: the shapes tuned for large images
-        fim_status s = choose_tile(j.kernel, j.dtype, limit, &ts, 0, 0);
+        fim_status s = choose_tile(j.kernel, j.dtype, use, limit, &ts, 0, 0);
         if (s != FIM_OK) return s;
-        const int n = j.kernel->n;
-        int rank = (n - 1) / 2;
-        if (j.percentile >= 0.0) rank = std::min(std::max((int)(j.percentile / 100.0 * (n - 1) + 0.5), 0), n - 1);
         Plan& p = plans[i];
-        s = make_plan(j.kernel, j.dtype, rank, j.w, j.h, ts, limit, &p);
+        s = make_plan(j.kernel, j.dtype, use, j.w, j.h, ts, limit, &p);
         if (s != FIM_OK) return s;
         p.in = j.in;
         p.out = j.out;

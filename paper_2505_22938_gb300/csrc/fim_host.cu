@@ -247,8 +247,10 @@ static int fill_vtab(const fim_kernel* k, int SP, int xmin, int* tab) {
     return units;
 }
 
-fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, const TileShape& ts, int smem_limit,
-                     Plan* p, int cta_threads, bool exact_ranks, int rank_hi) {
+fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, int h, const TileShape& ts,
+                     int smem_limit, Plan* p, int cta_threads) {
+    const int rank = use.rank, rank_hi = std::max(use.rank, use.rank_hi);
+    const bool exact_ranks = use.exact_ranks;
     memset(p, 0, sizeof(*p));
     p->dtype = dtype;
     p->w = w;
@@ -312,7 +314,6 @@ fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, con
     // a pivot ever takes, if those fit signed 16 bits (the packed slides then take one compare
     // instruction per pair of windows instead of three) or must (more than 65535 pixels); callers
     // whose targets vary per pixel or per kernel (exact_ranks) need N <= 65535.
-    if (rank_hi < rank) rank_hi = rank;
     p->rank_base = 0;
     p->s16 = N <= kMaxSignedRank ? 1 : 0;
     p->rel_max = p->s16 ? kMaxSignedRank : 65535;
@@ -610,13 +611,13 @@ static int resident_ctas(const Plan& p) {
     return std::max(1, std::min(std::min(by_regs, by_smem), std::min(2048 / p.threads, 32)));
 }
 
-bool small_image_shape(const fim_kernel* k, int dtype, int w, int h, int smem_limit, int cta_threads,
-                       bool exact_ranks, const TileShape& def, Plan* scratch, TileShape* out) {
+bool small_image_shape(const fim_kernel* k, int dtype, const PlanUse& use, int w, int h, int smem_limit,
+                       int cta_threads, const TileShape& def, Plan* scratch, TileShape* out) {
     if ((long long)w * h <= 0) return false;
     const int extent = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1;
     const int sms = device_sm_count();
     auto tiles = [&](const TileShape& c) { return (long long)((w + c.Tx - 1) / c.Tx) * ((h + c.Ty - 1) / c.Ty); };
-    if (make_plan(k, dtype, 0, 1, 1, def, smem_limit, scratch, cta_threads, exact_ranks) != FIM_OK) return false;
+    if (make_plan(k, dtype, use, 1, 1, def, smem_limit, scratch, cta_threads) != FIM_OK) return false;
     if (2 * tiles(def) >= (long long)sms * resident_ctas(*scratch)) return false;
     // kernels up to 65 pixels across: 32-wide tiles with 1-row bands first; larger kernels:
     // 8 bands of 2 or 4 rows (u8 256^2 r = 40 / 64 / 96: 35 / 49 / 70 us per call on 32x16
@@ -629,7 +630,7 @@ bool small_image_shape(const fim_kernel* k, int dtype, int w, int h, int smem_li
     const int nlist = big ? 2 : 3;
     for (int i = 0; i < nlist; ++i) {
         const TileShape& c = list[i];
-        if (make_plan(k, dtype, 0, 1, 1, c, smem_limit, scratch, cta_threads, exact_ranks) != FIM_OK ||
+        if (make_plan(k, dtype, use, 1, 1, c, smem_limit, scratch, cta_threads) != FIM_OK ||
             scratch->smem_bytes > smem_limit)
             continue;
         if (tiles(c) <= (long long)sms * resident_ctas(*scratch)) {
@@ -649,12 +650,12 @@ static bool parse_tile_env(TileShape* ts) {
     return true;
 }
 
-fim_status default_tile(const fim_kernel* k, int dtype, int rank, int smem_limit, int w, int h, int cta_threads,
-                        bool exact_ranks, bool (*fits)(Plan&), Plan* p, TileShape* ts) {
+fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, int w, int h,
+                        int cta_threads, bool (*fits)(Plan&), Plan* p, TileShape* ts) {
     const int extent = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1;
     const int pw = w > 0 ? w : 1, ph = h > 0 ? h : 1;
     auto valid = [&](const TileShape& c) {
-        return make_plan(k, dtype, rank, pw, ph, c, smem_limit, p, cta_threads, exact_ranks) == FIM_OK &&
+        return make_plan(k, dtype, use, pw, ph, c, smem_limit, p, cta_threads) == FIM_OK &&
                p->smem_bytes <= smem_limit && (!fits || fits(*p));
     };
     // Waves of the image's tiles on the resident CTAs of the plan in *p (a batch or an unknown size
@@ -681,7 +682,7 @@ fim_status default_tile(const fim_kernel* k, int dtype, int rank, int smem_limit
                                  {FIM_U16, 46, 59, {64, 64, 4, 2}, 2}};
     for (const Pref& c : prefs)
         if (c.dtype == dtype && c.lo <= extent && extent <= c.hi && valid(c.ts) && resident_ctas(*p) >= c.resident &&
-            (dtype == FIM_U8 || (p->codes > 0 && !exact_ranks)) && waves(c.ts) >= 1.25) {
+            (dtype == FIM_U8 || (p->codes > 0 && !use.exact_ranks)) && waves(c.ts) >= 1.25) {
             *ts = c.ts;
             return FIM_OK;
         }
@@ -742,15 +743,15 @@ fim_status default_tile(const fim_kernel* k, int dtype, int rank, int smem_limit
     return FIM_ERR_UNSUPPORTED;
 }
 
-fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape* ts, int w, int h,
-                       int cta_threads, bool exact_ranks, bool fixed_geometry) {
+fim_status choose_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, TileShape* ts, int w,
+                       int h, int cta_threads, bool fixed_geometry) {
     static const TileShape cands[] = {{32, 32, 2, 1}, {32, 32, 4, 1}, {64, 128, 8, 2}, {64, 64, 8, 2},
                                       {32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
     TileShape forced;
     if (parse_tile_env(&forced)) {  // explicit override (experiments, tuning)
         Plan* p = new (std::nothrow) Plan;
         if (!p) return FIM_ERR_OOM;
-        fim_status s = make_plan(k, dtype, 0, 1, 1, forced, smem_limit, p, cta_threads, exact_ranks);
+        fim_status s = make_plan(k, dtype, use, 1, 1, forced, smem_limit, p, cta_threads);
         const int bytes = p->smem_bytes;
         delete p;
         if (s != FIM_OK) return s;
@@ -764,7 +765,7 @@ fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape
     if ((cta_threads > 0 && tuned_lookup(k, dtype, &tuned, sc, cta_threads)) || tuned_lookup(k, dtype, &tuned, sc, 0)) {
         Plan* p = new (std::nothrow) Plan;
         if (!p) return FIM_ERR_OOM;
-        fim_status s = make_plan(k, dtype, 0, 1, 1, tuned, smem_limit, p, cta_threads, exact_ranks);
+        fim_status s = make_plan(k, dtype, use, 1, 1, tuned, smem_limit, p, cta_threads);
         delete p;
         if (s == FIM_OK) {
             *ts = tuned;
@@ -775,13 +776,13 @@ fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape
         Plan* p = new (std::nothrow) Plan;
         if (!p) return FIM_ERR_OOM;
         // (small images are told by the tiles a large one takes)
-        fim_status s = default_tile(k, dtype, 0, smem_limit, 0, 0, cta_threads, exact_ranks, nullptr, p, ts);
+        fim_status s = default_tile(k, dtype, use, smem_limit, 0, 0, cta_threads, nullptr, p, ts);
         TileShape small;
         if (s == FIM_OK && w > 0 && h > 0) {
-            if (small_image_shape(k, dtype, w, h, smem_limit, cta_threads, exact_ranks, *ts, p, &small))
+            if (small_image_shape(k, dtype, use, w, h, smem_limit, cta_threads, *ts, p, &small))
                 *ts = small;
             else
-                s = default_tile(k, dtype, 0, smem_limit, w, h, cta_threads, exact_ranks, nullptr, p, ts);
+                s = default_tile(k, dtype, use, smem_limit, w, h, cta_threads, nullptr, p, ts);
         }
         delete p;
         return s;
@@ -801,7 +802,7 @@ fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape
         inf->ok = false;
         Plan* p = new (std::nothrow) Plan;
         if (!p) return FIM_ERR_OOM;
-        const fim_status s = make_plan(k, dtype, 0, 1, 1, c, smem_limit, p, cta_threads, exact_ranks);
+        const fim_status s = make_plan(k, dtype, use, 1, 1, c, smem_limit, p, cta_threads);
         inf->ok = s == FIM_OK && p->smem_bytes <= smem_limit;
         inf->n = p->N;
         inf->om_smem = p->loc_om >= 0;
@@ -917,11 +918,12 @@ fim_status filter_rank(const void* in, void* out, int w, int h, size_t pitch, in
     if (smem_limit < 0) smem_limit = device_smem_limit();
     if (smem_limit <= 0) return FIM_ERR_CUDA;
     TileShape ts;
-    fim_status s = choose_tile(k, dtype, smem_limit, &ts, w, h);
+    const PlanUse use{rank};
+    fim_status s = choose_tile(k, dtype, use, smem_limit, &ts, w, h);
     if (s != FIM_OK) return s;
     Plan* p = new (std::nothrow) Plan;
     if (!p) return FIM_ERR_OOM;
-    s = make_plan(k, dtype, rank, w, h, ts, smem_limit, p);
+    s = make_plan(k, dtype, use, w, h, ts, smem_limit, p);
     if (s == FIM_OK) {
         p->in = in;
         p->out = out;
@@ -1087,21 +1089,18 @@ fim_status fim_percentiles(const void* in, void* const* outs, const double* perc
     static thread_local int smem_limit = -1;
     if (smem_limit < 0) smem_limit = device_smem_limit();
     if (smem_limit <= 0) return FIM_ERR_CUDA;
-    TileShape ts;
-    fim_status s = choose_tile(k, dtype, smem_limit, &ts, w, h);
-    if (s != FIM_OK) return s;
     int ranks[kMaxRanks];
     for (int i = 0; i < count; ++i)
         ranks[i] = std::min(std::max((int)floor(percentiles[i] / 100.0 * (k->n - 1) + 0.5), 0), k->n - 1);
+    // offset ranks (large footprints) must resolve every target's feasible ranks: a tile is chosen for
+    // all of them (chosen for one target, the tiles of disks from r = 114 on refused the quartiles)
+    const PlanUse use{*std::min_element(ranks, ranks + count), *std::max_element(ranks, ranks + count)};
+    TileShape ts;
+    fim_status s = choose_tile(k, dtype, use, smem_limit, &ts, w, h);
+    if (s != FIM_OK) return s;
     Plan* p = new (std::nothrow) Plan;
     if (!p) return FIM_ERR_OOM;
-    int rmin = ranks[0], rmax = ranks[0];
-    for (int i = 1; i < count; ++i) {
-        rmin = std::min(rmin, ranks[i]);
-        rmax = std::max(rmax, ranks[i]);
-    }
-    // offset ranks (large footprints) must resolve every target's feasible ranks
-    s = make_plan(k, dtype, rmin, w, h, ts, smem_limit, p, 0, false, rmax);
+    s = make_plan(k, dtype, use, w, h, ts, smem_limit, p);
     if (s == FIM_OK) {
         p->in = in;
         p->out = outs[0];
@@ -1135,11 +1134,12 @@ fim_status fim_median_radii(const void* in, void* const* outs, const fim_kernel*
     const fim_kernel* kb = kernels[big];
     TileShape ts;
     // the omnigram is narrowed from disk to disk with exact ranks: no rank offsets
-    fim_status s = choose_tile(kb, dtype, smem_limit, &ts, w, h, 0, true);
+    const PlanUse use{(kb->n - 1) / 2, -1, true};
+    fim_status s = choose_tile(kb, dtype, use, smem_limit, &ts, w, h);
     if (s != FIM_OK) return s;
     Plan* p = new (std::nothrow) Plan;
     if (!p) return FIM_ERR_OOM;
-    s = make_plan(kb, dtype, (kb->n - 1) / 2, w, h, ts, smem_limit, p, 0, true);
+    s = make_plan(kb, dtype, use, w, h, ts, smem_limit, p);
     // Targets run largest disk first, so that each footprint holds the next one and the tile can
     // narrow its omnigram from disk to disk. Every disk's tables (per-column vertical-slide
     // offsets, per-row horizontal offsets and spans) are relative to the window centre in the
@@ -1244,11 +1244,12 @@ fim_status fim_percentile_map(const void* in, void* out, const float* percentile
     if (smem_limit < 0) smem_limit = device_smem_limit();
     if (smem_limit <= 0) return FIM_ERR_CUDA;
     TileShape ts;
-    s = choose_tile(k, dtype, smem_limit, &ts, w, h, 0, true);  // a rank per pixel: exact ranks
+    const PlanUse use{(k->n - 1) / 2, -1, true};  // a rank per pixel: exact ranks
+    s = choose_tile(k, dtype, use, smem_limit, &ts, w, h);
     if (s != FIM_OK) return s;
     Plan* p = new (std::nothrow) Plan;
     if (!p) return FIM_ERR_OOM;
-    s = make_plan(k, dtype, (k->n - 1) / 2, w, h, ts, smem_limit, p, 0, true);
+    s = make_plan(k, dtype, use, w, h, ts, smem_limit, p);
     if (s == FIM_OK) {
         p->in = in;
         p->out = out;
@@ -1298,11 +1299,12 @@ fim_status fim_median_host(const void* in_host, void* out_host, int w, int h, si
     const int limit = device_smem_limit();
     if (limit <= 0) return FIM_ERR_CUDA;
     TileShape ts;
-    s = choose_tile(k, dtype, limit, &ts, w, h);
+    const PlanUse use{(k->n - 1) / 2};
+    s = choose_tile(k, dtype, use, limit, &ts, w, h);
     if (s != FIM_OK) return s;
     Plan* p = new (std::nothrow) Plan;
     if (!p) return FIM_ERR_OOM;
-    s = make_plan(k, dtype, (k->n - 1) / 2, w, h, ts, limit, p);
+    s = make_plan(k, dtype, use, w, h, ts, limit, p);
     if (s != FIM_OK) {
         delete p;
         return s;
@@ -1386,11 +1388,12 @@ fim_status fim_plan_info(const fim_kernel* k, fim_dtype dtype, int w, int h, int
     const int limit = device_smem_limit();
     if (limit <= 0) return FIM_ERR_CUDA;
     TileShape ts;
-    fim_status s = choose_tile(k, dtype, limit, &ts, w, h);
+    const PlanUse use{(k->n - 1) / 2};
+    fim_status s = choose_tile(k, dtype, use, limit, &ts, w, h);
     if (s != FIM_OK) return s;
     Plan* p = new (std::nothrow) Plan;
     if (!p) return FIM_ERR_OOM;
-    s = make_plan(k, dtype, (k->n - 1) / 2, w, h, ts, limit, p);
+    s = make_plan(k, dtype, use, w, h, ts, limit, p);
     if (s == FIM_OK) {
         if (tile_w) *tile_w = p->Tx;
         if (tile_h) *tile_h = p->Ty;

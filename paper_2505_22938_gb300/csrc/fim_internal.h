@@ -217,21 +217,27 @@ namespace fim {
 fim_status get_scratch(cudaStream_t stream, size_t bytes, unsigned char** out);
 fim_status release_scratch();
 int device_sm_count();
-// exact_ranks: the plan's targets vary per pixel or per kernel, so its ordinal image must hold
-// exact ranks (footprints up to 65535 pixels); otherwise larger footprints hold ranks relative to
-// the feasible ranks of the targets `rank` .. `rank_hi` (-1: `rank` alone).
-fim_status make_plan(const fim_kernel* k, int dtype, int rank, int w, int h, const TileShape& ts, int smem_limit,
-                     Plan* p, int cta_threads = 0, bool exact_ranks = false, int rank_hi = -1);
+// What a plan has to serve. A tile is chosen for the same use as it is planned for: a shape that
+// serves one target may not hold the ranks of several.
+struct PlanUse {
+    int rank;                  // target rank, the lowest of several
+    int rank_hi = -1;          // the highest (-1: `rank` alone)
+    bool exact_ranks = false;  // targets vary per pixel or per kernel: the ordinal image must hold exact
+                               // ranks (footprints up to 65535 pixels); otherwise larger footprints
+                               // hold ranks relative to the feasible ones of rank .. rank_hi
+};
+fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, int h, const TileShape& ts,
+                     int smem_limit, Plan* p, int cta_threads = 0);
 // Re-lays out a plan whose model is set so that the bracket MLP's parameters are staged in
 // shared memory; keeps them in device memory (off_model = -1) when they do not fit.
 fim_status plan_stage_model(Plan* p, int smem_limit);
 // Tile shape for an image of w x h (w or h <= 0: a batch, which fills the GPU like a large image).
-fim_status choose_tile(const fim_kernel* k, int dtype, int smem_limit, TileShape* ts, int w, int h,
-                       int cta_threads = 0, bool exact_ranks = false, bool fixed_geometry = false);
+fim_status choose_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, TileShape* ts, int w,
+                       int h, int cta_threads = 0, bool fixed_geometry = false);
 // The untuned tile shape. `fits` (may be null) is one more condition on a candidate's plan; p is
 // storage for trial plans.
-fim_status default_tile(const fim_kernel* k, int dtype, int rank, int smem_limit, int w, int h, int cta_threads,
-                        bool exact_ranks, bool (*fits)(Plan&), Plan* p, TileShape* ts);
+fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, int w, int h,
+                        int cta_threads, bool (*fits)(Plan&), Plan* p, TileShape* ts);
 int device_smem_limit();
 
 // Autotuner cache (fim_tune.cu).
@@ -261,8 +267,8 @@ void attach_tma(Plan& p);
 // to 65 pixels across: 32x8 with 4 bands, 32x16 with 4, 32x8 with 2; larger kernels: 32x16 and
 // 64x32 with 8 bands) whose tiles all fit in one wave of resident CTAs, in *out (true).
 // `scratch` is storage for trial plans.
-bool small_image_shape(const fim_kernel* k, int dtype, int w, int h, int smem_limit, int cta_threads,
-                       bool exact_ranks, const TileShape& def, Plan* scratch, TileShape* out);
+bool small_image_shape(const fim_kernel* k, int dtype, const PlanUse& use, int w, int h, int smem_limit,
+                       int cta_threads, const TileShape& def, Plan* scratch, TileShape* out);
 
 // Device launch (fim_tile.cu).
 fim_status launch_tile_kernel(Plan& p, cudaStream_t stream);

@@ -54,17 +54,17 @@ bool fits_array(fim::Plan& p) {
 // the autotuner's cache, whose lookup allocates. Trial plans and the chosen one are built in the
 // caller's storage.
 fim_status pick_plan(const fim_kernel* k, int dtype, int w, int h, int limit, fim::Plan* plan) {
-    const int rank = (k->n - 1) / 2;
+    const fim::PlanUse use{(k->n - 1) / 2};
     fim::TileShape ts, small;
     // the library's small-image rule, where its shape also fits the array
-    if (fim::default_tile(k, dtype, rank, limit, 0, 0, 0, false, nullptr, plan, &ts) == FIM_OK &&
-        fim::small_image_shape(k, dtype, w, h, limit, 0, false, ts, plan, &small) &&
-        fim::make_plan(k, dtype, rank, w, h, small, limit, plan) == FIM_OK && plan->smem_bytes <= limit &&
+    if (fim::default_tile(k, dtype, use, limit, 0, 0, 0, nullptr, plan, &ts) == FIM_OK &&
+        fim::small_image_shape(k, dtype, use, w, h, limit, 0, ts, plan, &small) &&
+        fim::make_plan(k, dtype, use, w, h, small, limit, plan) == FIM_OK && plan->smem_bytes <= limit &&
         fits_array(*plan))
         return FIM_OK;
-    fim_status s = fim::default_tile(k, dtype, rank, limit, w, h, 0, false, fits_array, plan, &ts);
+    fim_status s = fim::default_tile(k, dtype, use, limit, w, h, 0, fits_array, plan, &ts);
     if (s != FIM_OK) return s;
-    return fim::make_plan(k, dtype, rank, w, h, ts, limit, plan);
+    return fim::make_plan(k, dtype, use, w, h, ts, limit, plan);
 }
 
 bool overlap(const void* a, const void* b, size_t bytes) {

@@ -160,7 +160,7 @@ extern "C" fim_status fim_autotune(const void* in, void* out, int w, int h, size
     fim_status result = FIM_ERR_UNSUPPORTED;
     for (const TileShape& c : cands) {
         if (cta_threads != 0 && 2 * c.Tx * c.RB != cta_threads) continue;
-        if (make_plan(k, dtype, (k->n - 1) / 2, w, h, c, limit, p) != FIM_OK) continue;
+        if (make_plan(k, dtype, PlanUse{(k->n - 1) / 2}, w, h, c, limit, p) != FIM_OK) continue;
         p->in = in;
         p->out = out;
         p->pitch = (long long)pitch_bytes;

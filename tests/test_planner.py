@@ -1,0 +1,65 @@
+"""Plans of the entry points without a GPU: the library's host code runs against stand-ins of the
+CUDA calls (planner_probe.cpp, GB300's limits), and every call's plan is read back."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+CSRC = os.path.join(ROOT, "paper_2505_22938_gb300", "csrc")
+U8, U16, F32 = 0, 1, 2
+IN, OUT = 1 << 32, 1 << 36  # addresses only: nothing is read or written
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("planner") / "planner_probe.so")
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    cmd = ["g++", "-O1", "-std=c++17", "-w", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-x", "c++",
+           os.path.join(HERE, "planner_probe.cpp"), "-I", CSRC, "-I", os.path.join(ROOT, "include"), "-I", cuda,
+           "-o", so]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    dll = ctypes.CDLL(so)
+    dll.probe.restype = ctypes.c_longlong
+    return dll
+
+
+def disk(lib, r):
+    k = ctypes.c_void_p()
+    assert lib.fim_create_kernel_circle(r, ctypes.byref(k)) == 0
+    return k
+
+
+def ellipse(lib, a, b):
+    k = ctypes.c_void_p()
+    assert lib.fim_create_kernel_ellipse(a, b, ctypes.byref(k)) == 0
+    return k
+
+
+def plan(lib, *fields):
+    return [lib.probe(f.encode()) for f in fields]
+
+
+def outputs(n):
+    return (ctypes.c_void_p * n)(*[OUT + (i << 32) for i in range(n)])
+
+
+def percentiles(lib, k, dtype, w, h, pcts):
+    v = (ctypes.c_double * len(pcts))(*pcts)
+    return lib.fim_percentiles(ctypes.c_void_p(IN), outputs(len(pcts)), v, len(pcts), w, h,
+                               ctypes.c_size_t(w << dtype), dtype, k, 0, None)
+
+
+@pytest.mark.parametrize("dtype", [U8, U16, F32])
+@pytest.mark.parametrize("size", [(256, 256), (1537, 1021), (4096, 4096)])
+def test_quartiles_of_the_largest_disks_are_accepted(lib, dtype, size):
+    """The tile of several target ranks holds all of them: a footprint beyond 65535 pixels stores
+    ranks relative to the lowest target's, and the highest target's have to fit as well."""
+    for r in range(96, 129):
+        k = disk(lib, r)
+        assert percentiles(lib, k, dtype, *size, (25.0, 50.0, 75.0)) == 0, r
+        assert percentiles(lib, k, U16, *size, (5.0, 50.0, 95.0)) == 0 or r > 105, r
+        lib.fim_destroy_kernel(k)
