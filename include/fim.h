@@ -358,7 +358,9 @@ fim_status fim_plan_info(const fim_kernel* k, fim_dtype dtype, int w, int h, int
 /*
  * The filter keeps one device workspace per (device, stream) it has run on: the tile queue
  * counter and, for kernels whose footprint does not fit in shared memory, per-CTA buffers.
- * It grows on demand and lives until this call, which waits for the device and frees it.
+ * It grows on demand and lives until this call, which waits for the device and frees it. Calls
+ * that share one must not overlap on the GPU: a graph captured on a stream is not replayed beside
+ * other calls on that stream's workspace, and several host threads do not share cudaStreamPerThread.
  */
 fim_status fim_release_workspace(void);
 

@@ -139,7 +139,6 @@ fim_status get_scratch(cudaStream_t stream, size_t bytes, unsigned char** out) {
             return FIM_ERR_OOM;
         }
         b.bytes = want;
-        if (cudaMemsetAsync(b.ptr, 0, 256, stream) != cudaSuccess) return FIM_ERR_CUDA;  // the tile queue's header
     }
     *out = static_cast<unsigned char*>(b.ptr);
     return FIM_OK;

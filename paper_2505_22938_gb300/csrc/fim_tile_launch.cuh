@@ -1,7 +1,8 @@
 #pragma once
-// Single-image launches of the tile pipeline, for one kernel set KS (see process_tile): each CTA takes Tx x Ty output tiles from a device-side queue and filters them one
-// after the other (Sec. 3.3, Sec. 4.2). Included by one translation unit per KS, so that the
-// two sets of kernels compile in parallel.
+// Single-image launches of the tile pipeline, for one kernel set KS (see process_tile): each CTA
+// takes Tx x Ty output tiles from a device-side queue and filters them one after the other
+// (Sec. 3.3, Sec. 4.2). Included by one translation unit per KS, so that the two sets of kernels
+// compile in parallel.
 #include <atomic>
 
 #include "fim_tile_pipeline.cuh"
@@ -10,9 +11,8 @@ namespace fim {
 namespace {
 
 // Persistent CTAs: each takes tiles from the queue counter in the scratch header until none are
-// left. The workspace's header starts at zero and the last CTA to leave returns it to zero, so that
-// a launch needs no memset before it (u8 256^2 r = 4: a call 23.2 -> 21.7 us with the kept launch
-// set-up below).
+// left; the launch zeroes the counter first, so nothing of the queue is kept from one launch to the
+// next. A grid with a CTA for every tile needs no queue and no memset: CTA b takes tile b.
 template <int DT, int SHAPE, int W, int OG, int KS, int XT>
 __global__ void __launch_bounds__(1024, 1) tile_median_kernel(const __grid_constant__ Plan P) {
     __shared__ int s_tile;
@@ -25,18 +25,22 @@ __global__ void __launch_bounds__(1024, 1) tile_median_kernel(const __grid_const
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     TmaState tma{0u, 0};
     if (P.use_tma && tid == 0) mbar_init(reinterpret_cast<uint64_t*>(smem_dyn + P.off_misc + 34 * 4));
-    for (;;) {
-        if (tid == 0) s_tile = (int)atomicAdd(counter, 1u);
+    const bool queued = P.ntiles > (int)gridDim.x;
+    for (int tile = (int)blockIdx.x;;) {
+        if (queued && tid == 0) s_tile = (int)atomicAdd(counter, 1u);
         __syncthreads();
-        const int tile = s_tile;
+        if (queued) tile = s_tile;
         if (tile >= P.ntiles) break;
         stamp(P, tile, 0, G);
         process_tile<DT, SHAPE, W, OG, KS, XT>(P, P.tile0 + tile, gslice, G, &tma);
+        if (!queued) break;
     }
-    if (tid == 0 && atomicAdd(counter + 1, 1u) == gridDim.x - 1) {  // every CTA is past its last tile
-        counter[0] = 0;
-        counter[1] = 0;
-    }
+}
+
+// Zeroes the tile queue's counter before a launch of `grid` CTAs that takes its tiles from it.
+inline fim_status clear_queue(const Plan& p, int grid, cudaStream_t stream) {
+    if (p.ntiles <= grid) return FIM_OK;
+    return cudaMemsetAsync(p.scratch, 0, 16, stream) == cudaSuccess ? FIM_OK : FIM_ERR_CUDA;
 }
 
 // Set-up of a launch of this kernel: the shared-memory opt-in (the device's limit, once per device)
@@ -86,6 +90,8 @@ fim_status launch_typed(Plan& p, cudaStream_t stream) {
     if (s != FIM_OK) return s;
     p.scratch = scratch;
     attach_tma(p);
+    const fim_status cleared = clear_queue(p, grid, stream);
+    if (cleared != FIM_OK) return cleared;
     fn<<<grid, p.threads, p.smem_bytes, stream>>>(p);
     if (cudaGetLastError() != cudaSuccess) return FIM_ERR_CUDA;
     return FIM_OK;
@@ -108,8 +114,8 @@ fim_status launch_typed_fixed(Plan& p, unsigned char* scratch, size_t capacity, 
     if (!launch) return FIM_OK;
     p.scratch = scratch;
     attach_tma(p);
-    // (callers share this workspace by agreement alone: its queue is zeroed on every launch)
-    if (cudaMemsetAsync(scratch, 0, 16, stream) != cudaSuccess) return FIM_ERR_CUDA;
+    const fim_status cleared = clear_queue(p, grid, stream);
+    if (cleared != FIM_OK) return cleared;
     fn<<<grid, p.threads, p.smem_bytes, stream>>>(p);
     if (cudaGetLastError() != cudaSuccess) return FIM_ERR_CUDA;
     return FIM_OK;
