@@ -380,9 +380,9 @@ fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, 
     // coordinates hold. About 1.5 codes per pixel, in units the scan splits evenly (layout_plan
     // takes fewer where shared memory ends).
     p->codes = 0;
-    const bool lean = p->sort == kSortRadix && p->threads < 1024 && p->N >= 8000 && ts.Tx * ts.Ty >= 2048 &&
+    const bool lean = use.codes && p->sort == kSortRadix && p->threads < 1024 && p->N >= 8000 && ts.Tx * ts.Ty >= 2048 &&
                       p->threads >= (dtype == FIM_F32 ? 256 : 512);
-    if ((p->sort == kSortRadix16 || lean) && p->N <= 65535 && !p->wide) {
+    if (use.codes && (p->sort == kSortRadix16 || lean) && p->N <= 65535 && !p->wide) {
         const int unit = 256 * p->nwarps;
         p->code_bits = 10;
         p->codes = std::min(65536 / unit * unit - unit,
@@ -395,6 +395,7 @@ fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, 
         for (int v = 0; v < p->SH; v += 2) p->nsample2 += (p->frow[v] >> 16) - span_lo_host(p->frow[v]) + 1;
         if ((1 << p->code_bits) % p->threads != 0 || p->nsample == 0) p->codes = 0;
     }
+    p->xtab_words = use.table_words + use.row_tables * p->SH;
     // Placement. Tables, the ordinal image, medians and histograms always live in shared memory;
     // the omnigram, the radix keys and the radix position lists go to the CTA's global scratch
     // slice when shared memory cannot hold them (large kernels).
@@ -1132,8 +1133,16 @@ fim_status fim_median_radii(const void* in, void* const* outs, const fim_kernel*
     if (smem_limit <= 0) return FIM_ERR_CUDA;
     const fim_kernel* kb = kernels[big];
     TileShape ts;
-    // the omnigram is narrowed from disk to disk with exact ranks: no rank offsets
-    const PlanUse use{(kb->n - 1) / 2, -1, true};
+    // The omnigram is narrowed from disk to disk: exact ranks and exact order. The disks' tables (below)
+    // are part of every trial plan: chosen without them, the tiles filled shared memory so far that
+    // the tables put the omnigram in global scratch (u16 r = 68 .. 80, u8 r = 80 .. 86).
+    PlanUse use{(kb->n - 1) / 2, -1, true};
+    use.codes = false;
+    use.row_tables = count;
+    for (int i = 0; i < count; ++i) {
+        const int cols = kernels[i]->xmax - kernels[i]->xmin + 1, rows = kernels[i]->ymax - kernels[i]->ymin + 1;
+        use.table_words += 8 * (((cols + 1) / 2 + 1) / 2) + 3 * rows + 3;  // (3: alignment of the next disk's)
+    }
     fim_status s = choose_tile(kb, dtype, use, smem_limit, &ts, w, h);
     if (s != FIM_OK) return s;
     Plan* p = new (std::nothrow) Plan;
@@ -1191,9 +1200,8 @@ fim_status fim_median_radii(const void* in, void* const* outs, const fim_kernel*
             p->ranks[q] = (k->n - 1) / 2;
             p->outs[q] = outs[order[q]];
         }
+        if ((int)xt.size() > p->xtab_words) s = FIM_ERR_INTERNAL;
         p->xtab_words = (int)xt.size();
-        p->codes = 0;  // the omnigram is narrowed from disk to disk: exact order
-        s = layout_plan(p, smem_limit);
     }
     int* dx = nullptr;
     cudaStream_t st = (cudaStream_t)stream;

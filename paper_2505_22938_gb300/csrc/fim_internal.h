@@ -225,6 +225,10 @@ struct PlanUse {
     bool exact_ranks = false;  // targets vary per pixel or per kernel: the ordinal image must hold exact
                                // ranks (footprints up to 65535 pixels); otherwise larger footprints
                                // hold ranks relative to the feasible ones of rank .. rank_hi
+    bool codes = true;         // the omnigram may be sorted by equalised codes
+    // words of further tables in shared memory (several radii): their sum, and their tables of one
+    // word per box row
+    int table_words = 0, row_tables = 0;
 };
 fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, int h, const TileShape& ts,
                      int smem_limit, Plan* p, int cta_threads = 0);

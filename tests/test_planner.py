@@ -63,3 +63,23 @@ def test_quartiles_of_the_largest_disks_are_accepted(lib, dtype, size):
         assert percentiles(lib, k, dtype, *size, (25.0, 50.0, 75.0)) == 0, r
         assert percentiles(lib, k, U16, *size, (5.0, 50.0, 95.0)) == 0 or r > 105, r
         lib.fim_destroy_kernel(k)
+
+
+def radii(lib, dtype, w, h, rs):
+    ks = [disk(lib, r) for r in rs]
+    s = lib.fim_median_radii(ctypes.c_void_p(IN), outputs(len(rs)), (ctypes.c_void_p * len(rs))(*ks), len(rs), w, h,
+                             ctypes.c_size_t(w << dtype), dtype, 0, None)
+    for k in ks:
+        lib.fim_destroy_kernel(k)
+    return s
+
+
+@pytest.mark.parametrize("dtype,rs", [(U16, range(65, 81)), (U8, range(65, 89)), (F32, range(65, 83))])
+@pytest.mark.parametrize("size", [(1021, 763), (4096, 4096)])
+def test_several_radii_keep_their_omnigram_in_shared_memory(lib, dtype, rs, size):
+    """The disks' tables are part of the plan the tile is chosen by; float keys keep the 16-bit first pass
+    (a plan that cannot sort by codes has no cheaper sort to fall back from)."""
+    for r in rs:
+        assert radii(lib, dtype, *size, (r // 2, r)) == 0
+        assert plan(lib, "spilled", "codes") == [0, 0], r
+        assert dtype != F32 or plan(lib, "sort") == [3], r
