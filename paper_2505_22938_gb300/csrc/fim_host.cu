@@ -1202,6 +1202,7 @@ fim_status fim_median_radii(const void* in, void* const* outs, const fim_kernel*
         }
         if ((int)xt.size() > p->xtab_words) s = FIM_ERR_INTERNAL;
         p->xtab_words = (int)xt.size();
+        if (s == FIM_OK) s = layout_plan(p, smem_limit);  // (without the words kept for alignment)
     }
     int* dx = nullptr;
     cudaStream_t st = (cudaStream_t)stream;

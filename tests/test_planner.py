@@ -83,3 +83,9 @@ def test_several_radii_keep_their_omnigram_in_shared_memory(lib, dtype, rs, size
         assert radii(lib, dtype, *size, (r // 2, r)) == 0
         assert plan(lib, "spilled", "codes") == [0, 0], r
         assert dtype != F32 or plan(lib, "sort") == [3], r
+
+
+def test_several_radii_keep_their_resident_ctas(lib):
+    """The words kept for the alignment of the disks' tables are given back before the launch."""
+    assert radii(lib, U8, 3047, 5420, (15, 30)) == 0
+    assert plan(lib, "threads", "resident") == [256, 4]
