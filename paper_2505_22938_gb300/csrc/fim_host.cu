@@ -670,7 +670,12 @@ fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int 
     //    4096^2 against the one-CTA shapes: u8 r = 24 / 32 / 40 / 48 / 56 1.47x / 1.38x / 1.28x /
     //    1.22x / 1.13x, f32 r = 16 / 20 / 24 / 32 / 40 / 48 1.13x / 1.25x / 1.21x / 1.11x / 1.08x /
     //    1.04x, u16 r = 24 / 27 1.07x / 1.04x; u8 r = 64 and f32 r = 56, one CTA per SM, 1.0 and 0.9x.
-    //    An image of little over one wave of them has nothing to overlap.
+    //    An image of little over one wave of them has nothing to overlap, and up to 45 pixels across,
+    //    where rule 2's tiles are a quarter of the size, the last wave costs more than that below three
+    //    waves (f32 r = 20 at 2000x1500, 2.5 waves 531 us against 439, at 2500x1800, 3.8 waves 529
+    //    against 599; u8 r = 17 at 2.7 waves 259 against 244, at 3.9 327 against 373). Several target
+    //    ranks pay for one sort only, so that rule 2's smaller tiles are ahead for float data as well
+    //    (quartiles r = 20 at 3000x2000 1582 against 1427 us, 2000x1500 1128 against 768).
     struct Pref {
         int dtype, lo, hi;  // kernel extents
         TileShape ts;
@@ -680,19 +685,23 @@ fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int 
                                  {FIM_U8, 68, 115, {64, 48, 4, 2}, 2}, {FIM_U8, 68, 115, {64, 40, 4, 2}, 2},
                                  {FIM_F32, 29, 34, {64, 64, 2, 2}, 3}, {FIM_F32, 35, 99, {64, 64, 4, 2}, 2},
                                  {FIM_U16, 46, 59, {64, 64, 4, 2}, 2}};
+    const bool several = use.rank_hi > use.rank;
     for (const Pref& c : prefs)
         if (c.dtype == dtype && c.lo <= extent && extent <= c.hi && valid(c.ts) && resident_ctas(*p) >= c.resident &&
-            (dtype == FIM_U8 || (p->codes > 0 && !use.exact_ranks)) && waves(c.ts) >= 1.25) {
+            (dtype == FIM_U8 || (p->codes > 0 && !use.exact_ranks)) && waves(c.ts) >= (extent <= 45 ? 3.0 : 1.25) &&
+            !(several && dtype == FIM_F32 && extent <= 45)) {
             *ts = c.ts;
             return FIM_OK;
         }
     // 2. Small kernels: 32-column tiles in CTAs of 128 or 256 threads, many per SM (the footprint, and
     //    so every scan, shrinks with the tile; 16-bit data then sorts by radix passes).
-    //    (u16 r = 18 / 22 32x64 1.04x / 1.07x over 32x32, both with four bands, on several waves.)
+    //    (u16 r = 18 / 22 32x64 1.04x / 1.07x over 32x32, both with four bands, at 4096^2, r = 20 equal at
+    //    2500x1800, 5.0 waves, and 389 us against 312 at 2000x1500; the quartiles 1353 against 1221 at
+    //    3000x2000.)
     static const TileShape small[] = {{32, 32, 2, 1}, {32, 64, 4, 1}, {32, 32, 4, 1}};
     if (extent <= 45)
         for (int i = extent <= 33 ? 0 : 1; i < 3; ++i)
-            if (valid(small[i]) && (i != 1 || (dtype == FIM_U16 && waves(small[i]) >= 2.0))) {
+            if (valid(small[i]) && (i != 1 || (dtype == FIM_U16 && !several && waves(small[i]) >= 5.0))) {
                 *ts = small[i];
                 return FIM_OK;
             }
@@ -703,25 +712,38 @@ fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int 
     //    u16 r = 72 / 88 64x96 / 64x48 1.10x / 1.39x over 64x64, f32 r = 72 1.14x, u8 r = 92 64x56
     //    1.52x; f32 400x719 r = 51 64x48 2.3x over 64x128; in global scratch the omnigram's entries
     //    cost each scan an L2 access).
+    //    One wave takes as long as its slowest tiles, those of the last row, whose windows below the image
+    //    hold its last row many times: where the best height's tiles all run at once, the one of least
+    //    rows, counted with those below the image, of which that is true (u8 587x410 r = 94: 64x48, 90
+    //    tiles, 168 us, 64x32, 130 tiles, 139; f32 956x539 r = 117 64x96 804, 64x64 580; u16 858x447
+    //    r = 43 64x48, 33 rows below, 140, 64x56, one row below, 120). `whole`: waves are counted whole.
     static const int heights[] = {128, 112, 96, 88, 80, 72, 64, 56, 48, 40, 32};
-    auto cheapest = [&](double own, bool spilled, int least, bool coded) {
+    auto cheapest = [&](double own, bool spilled, int least, bool coded, bool whole) {
         double best = 0.0;
+        int one = 0;  // rows of the best height so far, if it runs in one wave
         for (int ty : heights) {
             const TileShape c{64, ty, 8, 2};
             if (ty < least || !valid(c) || (p->loc_om < 0) != spilled || (coded && p->codes == 0)) continue;
             double cost = (ty + own) / ty * (p->wide ? 1.08 : 1.0);
+            int rows = 0;
             if (w > 0 && h > 0) {
                 const double n = (double)((w + 63) / 64) * ((h + ty - 1) / ty) / device_sm_count();
-                cost *= std::max(ceil(n), n + 0.6) * ty;
+                cost *= (whole ? ceil(n) : std::max(ceil(n), n + 0.6)) * ty;
+                if (n <= 1.0) rows = 2 * ty - 1 - (h - 1) % ty;
             }
-            if (best == 0.0 || cost < best) {
-                best = cost;
+            if (one > 0 && rows > 0 ? rows <= one : best == 0.0 || cost < best) {
+                best = best == 0.0 ? cost : std::min(best, cost);
+                one = rows;
                 *ts = c;
             }
         }
         return best > 0.0;
     };
-    if (cheapest(0.27 * extent, false, w > 0 && h > 0 && (long long)w * h < 64LL * 48 * 304 ? 32 : 48, false)) return FIM_OK;
+    // (heights below 48 only where the image has less than two waves of 64x48)
+    auto below = [&](double n, int ty) {
+        return w > 0 && h > 0 && (double)w * h < n * device_sm_count() * 64.0 * ty;
+    };
+    if (cheapest(0.27 * extent, false, below(2.0, 48) ? 32 : 48, false, false)) return FIM_OK;
     const TileShape low{64, 40, 4, 2};
     if (dtype == FIM_U8 && valid(low) && p->loc_om >= 0) {  // (u8 r = 96: 1.31x over the spilled shapes)
         *ts = low;
@@ -731,9 +753,25 @@ fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int 
     //    64x128), otherwise by cost, which for 8-bit and 16-bit data is nearly proportional to the
     //    rows up to r = 96 (u16: 64x64 354k, 64x128 694k cycles) and less so above (r = 128: 64x64
     //    587k, 64x88 696k), and for a float radix sort is not (r = 100: 64x128 1.2x over 64x64;
-    //    r = 128: 64x88 1.18x over 64x64): at least 88 rows where they fit.
-    if (dtype == FIM_F32 && (cheapest(3.0, true, 64, true) || cheapest(32.0, true, 88, false))) return FIM_OK;
-    if (cheapest(std::max(3.0, 0.9 * (extent - 193)), true, 64, false)) return FIM_OK;
+    //    r = 128: 64x88 1.18x over 64x64): at least 88 rows where they fit. On images of less than three
+    //    waves of 64x64 most tiles leave the image, and those of 8-bit and 16-bit data cost more than in
+    //    proportion to their rows (u16 1537x1021 r = 128: 64x64 400 tiles 1078 us, 64x88 300 tiles 1668;
+    //    u8 r = 117 920, 1553; 1139x837 r = 108 .. 128 1.2-1.5x; but 1325x1092 r = 107 0.85x): 64x64, or
+    //    one wave of slightly taller tiles (u16 590x1036 r = 97: 64x72, 150 tiles, 283 us, 64x64 433). Float
+    //    tiles' waves are counted whole below four (1537x1021 r = 117: 64x88, two waves, 1295 us, 64x96,
+    //    two waves, 1544, 64x64 1487; several radii r = 88 64x112 2090, 64x88 1468).
+    const bool few = below(4.0, 64);
+    if (dtype == FIM_F32 && (cheapest(3.0, true, 64, true, false) || cheapest(32.0, true, few ? 64 : 88, false, few)))
+        return FIM_OK;
+    auto takes = [&](int ty, int waves_most) {  // 64 columns by ty rows, if that is few enough tiles
+        const TileShape c{64, ty, 8, 2};
+        const long long tiles = (long long)((w + 63) / 64) * ((h + ty - 1) / ty);
+        if (w <= 0 || h <= 0 || tiles > (long long)waves_most * device_sm_count() || !valid(c)) return false;
+        *ts = c;
+        return true;
+    };
+    if (takes(64, 1) || takes(72, 1) || takes(80, 1) || takes(64, 3)) return FIM_OK;
+    if (cheapest(std::max(3.0, 0.9 * (extent - 193)), true, 64, false, false)) return FIM_OK;
     static const TileShape last[] = {{32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
     for (const TileShape& c : last)
         if (valid(c)) {

@@ -89,3 +89,26 @@ def test_several_radii_keep_their_resident_ctas(lib):
     """The words kept for the alignment of the disks' tables are given back before the launch."""
     assert radii(lib, U8, 3047, 5420, (15, 30)) == 0
     assert plan(lib, "threads", "resident") == [256, 4]
+
+
+def median(lib, k, dtype, w, h):
+    return lib.fim_median(ctypes.c_void_p(IN), ctypes.c_void_p(OUT), w, h, ctypes.c_size_t(w << dtype), dtype, k, 0,
+                          None)
+
+
+@pytest.mark.parametrize("dtype,r,size,tile", [
+    (U8, 94, (587, 410), (64, 32)),       # all tiles at once: the height of least rows, not a taller one
+    (F32, 117, (956, 539), (64, 64)),
+    (U16, 43, (858, 447), (64, 56)),      # rows below the image count as well
+    (U16, 128, (1537, 1021), (64, 64)),   # few waves of border tiles, omnigram in global scratch
+    (U16, 97, (590, 1036), (64, 72)),
+    (F32, 20, (2000, 1500), (32, 32)),    # less than three waves of the larger tiles
+    (U16, 20, (2000, 1500), (32, 32)),
+    (F32, 20, (4096, 4096), (64, 64)),
+    (U16, 20, (4096, 4096), (32, 64)),
+])
+def test_tiles_of_images_of_few_waves(lib, dtype, r, size, tile):
+    k = disk(lib, r)
+    assert median(lib, k, dtype, *size) == 0
+    assert tuple(plan(lib, "Tx", "Ty")) == tile
+    lib.fim_destroy_kernel(k)
