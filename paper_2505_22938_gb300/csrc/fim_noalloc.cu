@@ -19,7 +19,7 @@
 namespace {
 
 // Workspace of every fim_median_noalloc call on this device: a 256-byte header (the tile queue
-// counter, cleared before each launch) followed by the per-CTA buffers of large kernels.
+// counter, set by each launch) followed by the per-CTA buffers of large kernels.
 static __device__ __align__(256) unsigned char g_noalloc_workspace[FIM_NOALLOC_WORKSPACE_BYTES];
 
 constexpr int kMaxDevices = 64;
