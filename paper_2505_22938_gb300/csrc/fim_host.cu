@@ -399,7 +399,30 @@ fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, 
     // Placement. Tables, the ordinal image, medians and histograms always live in shared memory;
     // the omnigram, the radix keys and the radix position lists go to the CTA's global scratch
     // slice when shared memory cannot hold them (large kernels).
-    return layout_plan(p, smem_limit);
+    const bool full = p->sort == kSortRadix16;
+    fim_status s = layout_plan(p, smem_limit);
+    // Beside a sort by codes the exact sort may have to give up its 16-bit pass, which pays where a
+    // quarter of the tiles have their box inside the image, as the sort by codes asks (cycles per
+    // tile at r = 64: by codes 83k, 16-bit and two 8-bit passes 227k, four 8-bit passes about 280k;
+    // f32 448x261 r = 92, 4 of 63 tiles inside, 251 us with codes, 207 without). (1 x 1: any size.)
+    if (s == FIM_OK && full && p->sort == kSortRadix && p->codes > 0 && (w > 1 || h > 1)) {
+        auto inside = [](int first, int step, int box, int size) {  // tiles whose box lies in [0, size)
+            const int a = first < 0 ? (step - 1 - first) / step : 0, b = size - box - first;
+            return b < 0 ? 0 : std::max(0, b / step - a + 1);
+        };
+        if (4LL * inside(p->xmin, Tx, S, w) * inside(p->ymin, Ty, p->SH, h) < (long long)p->tiles_x * p->tiles_y) {
+            const int coded = p->codes, om = p->loc_om;
+            p->codes = 0;
+            p->sort = kSortRadix16;
+            s = layout_plan(p, smem_limit);
+            if (s != FIM_OK || (p->loc_om < 0 && om >= 0)) {  // not at the price of the omnigram's place
+                p->codes = coded;
+                p->sort = kSortRadix16;
+                s = layout_plan(p, smem_limit);
+            }
+        }
+    }
+    return s;
 }
 
 fim_status plan_stage_model(Plan* p, int smem_limit) {
@@ -617,7 +640,7 @@ bool small_image_shape(const fim_kernel* k, int dtype, const PlanUse& use, int w
     const int extent = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1;
     const int sms = device_sm_count();
     auto tiles = [&](const TileShape& c) { return (long long)((w + c.Tx - 1) / c.Tx) * ((h + c.Ty - 1) / c.Ty); };
-    if (make_plan(k, dtype, use, 1, 1, def, smem_limit, scratch, cta_threads) != FIM_OK) return false;
+    if (make_plan(k, dtype, use, w, h, def, smem_limit, scratch, cta_threads) != FIM_OK) return false;
     if (2 * tiles(def) >= (long long)sms * resident_ctas(*scratch)) return false;
     // kernels up to 65 pixels across: 32-wide tiles with 1-row bands first; larger kernels:
     // 8 bands of 2 or 4 rows (u8 256^2 r = 40 / 64 / 96: 35 / 49 / 70 us per call on 32x16
@@ -630,7 +653,7 @@ bool small_image_shape(const fim_kernel* k, int dtype, const PlanUse& use, int w
     const int nlist = big ? 2 : 3;
     for (int i = 0; i < nlist; ++i) {
         const TileShape& c = list[i];
-        if (make_plan(k, dtype, use, 1, 1, c, smem_limit, scratch, cta_threads) != FIM_OK ||
+        if (make_plan(k, dtype, use, w, h, c, smem_limit, scratch, cta_threads) != FIM_OK ||
             scratch->smem_bytes > smem_limit)
             continue;
         if (tiles(c) <= (long long)sms * resident_ctas(*scratch)) {

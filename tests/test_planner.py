@@ -112,3 +112,11 @@ def test_tiles_of_images_of_few_waves(lib, dtype, r, size, tile):
     assert median(lib, k, dtype, *size) == 0
     assert tuple(plan(lib, "Tx", "Ty")) == tile
     lib.fim_destroy_kernel(k)
+
+
+@pytest.mark.parametrize("size,sort,codes", [((448, 261), 3, 0), ((553, 296), 3, 0), ((3000, 2000), 2, 1)])
+def test_float_images_of_border_tiles_keep_the_16_bit_pass(lib, size, sort, codes):
+    k = disk(lib, 92)
+    assert median(lib, k, F32, *size) == 0
+    assert plan(lib, "sort", "codes", "spilled") == [sort, codes, 0]
+    lib.fim_destroy_kernel(k)
