@@ -336,14 +336,21 @@ fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, 
     // that corner belongs to the footprint (then it would be a real entry, and a member of some
     // window). The disk test multiplies them by twice the window centre's coordinates as signed
     // bytes (centres in [-63, 64]); 128-pixel tiles meet that with the origin at (S - 1) / 2,
-    // which boxes below 256 pixels allow.
+    // which boxes below 256 pixels allow. A disk on a tile that does not (r = 64 on 128 rows) takes the
+    // span test, which has no such limit and keeps the 8-bit coordinates (with 16-bit ones the
+    // omnigram went to global scratch); several radii, whose disks the test's table does not hold,
+    // take 16-bit coordinates.
     const bool corner = span_lo_host(p->frow[0]) == 0;
     p->cx0 = S < 256 ? (S - 1) / 2 : S / 2;
     p->cy0 = p->SH < 256 ? (p->SH - 1) / 2 : p->SH / 2;
     const int px0 = -k->xmin - p->cx0, py0 = -k->ymin - p->cy0;  // the tile's first window centre
     const bool far = p->shape == kShapeDisk &&
                      (px0 < -63 || px0 + Tx - 1 > 64 || py0 < -63 || py0 + Ty - 1 > 64);
-    p->wide = (p->S > 256 || p->SH > 256 || (p->S == 256 && p->SH == 256 && corner) || far) ? 1 : 0;
+    p->wide = (p->S > 256 || p->SH > 256 || (p->S == 256 && p->SH == 256 && corner)) ? 1 : 0;
+    if (far && !p->wide) {
+        if (use.row_tables > 0) p->wide = 1;
+        else p->shape = kShapeSpans;
+    }
     p->div_magic = (unsigned)(((1ull << 32) + (unsigned)S - 1) / (unsigned)S);
     int hs = 0;
     const int rel_top = std::min(p->N - 1, p->rel_max);
@@ -679,7 +686,7 @@ fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int 
     const int pw = w > 0 ? w : 1, ph = h > 0 ? h : 1;
     auto valid = [&](const TileShape& c) {
         return make_plan(k, dtype, use, pw, ph, c, smem_limit, p, cta_threads) == FIM_OK &&
-               p->smem_bytes <= smem_limit && (!fits || fits(*p));
+               p->smem_bytes <= smem_limit && p->shape == k->shape && (!fits || fits(*p));
     };
     // Waves of the image's tiles on the resident CTAs of the plan in *p (a batch or an unknown size
     // counts as large).

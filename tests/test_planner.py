@@ -120,3 +120,15 @@ def test_float_images_of_border_tiles_keep_the_16_bit_pass(lib, size, sort, code
     assert median(lib, k, F32, *size) == 0
     assert plan(lib, "sort", "codes", "spilled") == [sort, codes, 0]
     lib.fim_destroy_kernel(k)
+
+
+def test_disk_of_256_box_rows_keeps_8_bit_coordinates(lib, monkeypatch):
+    """r = 64 on 128 rows: the disk test's signed bytes do not reach every window centre."""
+    monkeypatch.setenv("FIM_TILE", "64,128,8,2")
+    k = disk(lib, 64)
+    for dtype in (U8, U16, F32):
+        assert median(lib, k, dtype, 2000, 1500) == 0
+        assert plan(lib, "wide", "spilled") == [0, 0]
+        assert radii(lib, dtype, 2000, 1500, (30, 64)) == 0
+        assert plan(lib, "wide") == [1]
+    lib.fim_destroy_kernel(k)
