@@ -811,10 +811,95 @@ fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int 
     return FIM_ERR_UNSUPPORTED;
 }
 
-fim_status choose_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, TileShape* ts, int w,
-                       int h, int cta_threads, bool fixed_geometry) {
+// Tile of the learned bracket and its training rows. A model is trained on one tile's features, and a
+// saved one outlives changes to the plans: the rule rests on sizes of its own (those of the layout the
+// first models were trained on), not on what a plan of this library takes today.
+// Kernels up to 33 pixels across 32x32 tiles with two bands, up to 45 across with four, up to 64 across
+// 64x64, beyond 64x128: the first shape that fits; a later one of at least 64x64 that keeps the
+// omnigram in shared memory before one that spills it; for 16-bit data beyond 65535 pixels the first
+// shape within, if that is of at least 64x64.
+static fim_status bracket_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, int cta_threads,
+                               TileShape* ts) {
     static const TileShape cands[] = {{32, 32, 2, 1}, {32, 32, 4, 1}, {64, 128, 8, 2}, {64, 64, 8, 2},
                                       {32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
+    const int ncands = (int)(sizeof(cands) / sizeof(cands[0]));
+    const int ncols = k->xmax - k->xmin + 1, nrows = k->ymax - k->ymin + 1;
+    const int extent = std::max(ncols, nrows);
+    struct Sizes {
+        bool ok, om_smem;
+        int64_t n;
+    };
+    auto sizes = [&](const TileShape& c) {
+        Sizes z{false, false, 0};
+        const int S = c.Tx + ncols - 1, SH = c.Ty + nrows - 1, threads = std::max(2 * c.Tx * c.RB, cta_threads);
+        if (S > kMaxSide || SH > kMaxSide || threads > 1024) return z;
+        int SP = (S + 1) & ~1;
+        if ((SP / 2) % 2 == 0) SP += 2;
+        bool corner = false;
+        for (int v = 0; v < SH; ++v) {  // the footprint's rows (Fig. 10)
+            int lo = 1 << 30, hi = -(1 << 30);
+            for (int i = std::max(0, v - c.Ty + 1); i <= std::min(nrows - 1, v); ++i) {
+                lo = std::min(lo, k->rlo[i]);
+                hi = std::max(hi, k->rhi[i]);
+            }
+            z.n += c.Tx + hi - lo;
+            if (v == 0) corner = lo == k->xmin;
+        }
+        if (z.n - k->n > 65535) return z;
+        const bool wide = S > 256 || SH > 256 || (S == 256 && SH == 256 && corner);
+        const int64_t tab = align16(8 * ncols) + align16(8 * nrows) + align16(4 * nrows) + align16(4 * SH) + 256;
+        const int64_t om = align16((size_t)z.n * (wide ? 4 : 2));
+        const int64_t hists = z.n < 4 * (int64_t)k->n ? 1 : std::min(threads / 32, c.RB * c.G);
+        const int64_t solve = align16((size_t)SP * SH * 2) + align16((size_t)c.Tx * c.Ty * 2) + hists * 1024;
+        int64_t need = 0;
+        if (dtype == FIM_U8 || (dtype == FIM_U16 && threads >= 1024)) {
+            const int64_t region = std::max<int64_t>(dtype == FIM_U8 ? 1024 : 131072, solve);
+            z.om_smem = !wide && tab + om + region <= smem_limit;
+            need = tab + region + (z.om_smem ? om : 0);
+        } else {
+            const int64_t keys = align16((size_t)S * SH * 4), digits = align16((size_t)S * SH);
+            const int64_t hist = align16((size_t)(threads / 32) * (kSortBins + 1) * 4);
+            need = smem_limit + 1;
+            for (int64_t bins : {131072, 0}) {
+                if (bins > 0 && (dtype != FIM_F32 || threads < 1024)) continue;
+                for (int mode = wide ? 2 : 0; mode < 3 && need > smem_limit; ++mode) {
+                    const int64_t list = mode == 0 ? om : dtype == FIM_F32 ? digits : mode == 1 ? om : 0;
+                    z.om_smem = mode < 2;
+                    need = tab + (mode < 2 ? om : 0) +
+                           std::max((mode == 0 ? keys : 0) + std::max(list + hist, bins), solve);
+                }
+            }
+        }
+        z.ok = need <= smem_limit;
+        return z;
+    };
+    int pick = extent <= 33 ? 0 : (extent <= 45 ? 1 : (extent >= 65 ? 2 : 3));
+    while (pick < ncands && !sizes(cands[pick]).ok) ++pick;
+    if (pick == ncands) return FIM_ERR_UNSUPPORTED;
+    const int first = pick;
+    const Sizes f = sizes(cands[first]);
+    for (int i = first + 1; i < ncands && pick == first && !f.om_smem; ++i) {
+        const Sizes z = sizes(cands[i]);
+        if (z.ok && z.om_smem && cands[i].Tx * cands[i].Ty >= 4096) pick = i;
+    }
+    for (int i = first + 1; i < ncands && pick == first && dtype == FIM_U16 && f.n > 65535; ++i) {
+        const Sizes z = sizes(cands[i]);
+        if (!z.ok || z.n > 65535) continue;
+        if (cands[i].Tx * cands[i].Ty >= 4096) pick = i;
+        break;
+    }
+    Plan* p = new (std::nothrow) Plan;
+    if (!p) return FIM_ERR_OOM;
+    // (should a plan of this library not fit where those sizes did: the next shape whose plan does)
+    while (pick < ncands && make_plan(k, dtype, use, 1, 1, cands[pick], smem_limit, p, cta_threads) != FIM_OK) ++pick;
+    delete p;
+    if (pick == ncands) return FIM_ERR_UNSUPPORTED;
+    *ts = cands[pick];
+    return FIM_OK;
+}
+
+fim_status choose_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, TileShape* ts, int w,
+                       int h, int cta_threads, bool fixed_geometry) {
     TileShape forced;
     if (parse_tile_env(&forced)) {  // explicit override (experiments, tuning)
         Plan* p = new (std::nothrow) Plan;
@@ -855,53 +940,18 @@ fim_status choose_tile(const fim_kernel* k, int dtype, const PlanUse& use, int s
         delete p;
         return s;
     }
-    // Fixed geometry (training rows and the learned bracket, whose features and labels depend on the
-    // tile): kernels up to 33 pixels across 32x32 tiles with two bands, up to 45 across with four, up
-    // to 64 across 64x64, beyond 64x128; a shape of at least 64x64 that keeps the omnigram in shared
-    // memory before one that spills it; for 16-bit data the first exact-rank shape of at least 64x64.
-    const int extent = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1;
-    const int first = extent <= 33 ? 0 : (extent <= 45 ? 1 : (extent >= 65 ? 2 : 3));
-    struct Info {
-        bool ok;
-        int n;
-        bool om_smem;
-    };
-    auto probe = [&](const TileShape& c, Info* inf) {
-        inf->ok = false;
-        Plan* p = new (std::nothrow) Plan;
-        if (!p) return FIM_ERR_OOM;
-        const fim_status s = make_plan(k, dtype, use, 1, 1, c, smem_limit, p, cta_threads);
-        inf->ok = s == FIM_OK && p->smem_bytes <= smem_limit;
-        inf->n = p->N;
-        inf->om_smem = p->loc_om >= 0;
-        delete p;
-        return FIM_OK;
-    };
-    const int ncands = (int)(sizeof(cands) / sizeof(cands[0]));
-    int i0 = -1;
-    Info f{};
-    for (int i = first; i < ncands && i0 < 0; ++i) {
-        if (probe(cands[i], &f) != FIM_OK) return FIM_ERR_OOM;
-        if (f.ok) i0 = i;
-    }
-    if (i0 < 0) return FIM_ERR_UNSUPPORTED;
-    Info g{};
-    int pick = i0;
-    if (!f.om_smem)
-        for (int i = i0 + 1; i < ncands && pick == i0; ++i) {
-            if (probe(cands[i], &g) != FIM_OK) return FIM_ERR_OOM;
-            if (g.ok && g.om_smem && cands[i].Tx * cands[i].Ty >= 4096) pick = i;
-        }
-    if (pick == i0 && dtype == FIM_U16 && f.n > 65535)
-        for (int i = i0 + 1; i < ncands; ++i) {
-            if (probe(cands[i], &g) != FIM_OK) return FIM_ERR_OOM;
-            if (g.ok && g.n <= 65535) {
-                if (cands[i].Tx * cands[i].Ty >= 4096) pick = i;
-                break;
-            }
-        }
-    *ts = cands[pick];
-    return FIM_OK;
+    return bracket_tile(k, dtype, use, smem_limit, cta_threads, ts);
+}
+
+// The bracket's features, labels and calibrated width depend on the tile, so training rows and learned
+// launches take the same one, the large-image shape whatever the image size. The sort is exact: the
+// features are values and ranks at places of the sorted footprint.
+fim_status bracket_plan(const fim_kernel* k, int dtype, int w, int h, int smem_limit, Plan* p) {
+    PlanUse use{(k->n - 1) / 2};
+    use.codes = false;
+    TileShape ts;
+    const fim_status s = choose_tile(k, dtype, use, smem_limit, &ts, 0, 0, 0, true);
+    return s != FIM_OK ? s : make_plan(k, dtype, use, w, h, ts, smem_limit, p);
 }
 
 }  // namespace fim

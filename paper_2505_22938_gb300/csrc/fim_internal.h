@@ -235,6 +235,8 @@ fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, 
 // Re-lays out a plan whose model is set so that the bracket MLP's parameters are staged in
 // shared memory; keeps them in device memory (off_model = -1) when they do not fit.
 fim_status plan_stage_model(Plan* p, int smem_limit);
+// Plan of the learned bracket's launches and of its training rows.
+fim_status bracket_plan(const fim_kernel* k, int dtype, int w, int h, int smem_limit, Plan* p);
 // Tile shape for an image of w x h (w or h <= 0: a batch, which fills the GPU like a large image).
 fim_status choose_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, TileShape* ts, int w,
                        int h, int cta_threads = 0, bool fixed_geometry = false);

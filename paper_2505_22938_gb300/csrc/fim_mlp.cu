@@ -258,19 +258,10 @@ fim_status run_filter(const void* in, void* out, int w, int h, size_t pitch, int
     if (pitch < (size_t)w * es || pitch % es != 0) return FIM_ERR_INVALID_ARG;
     const int limit = device_smem_limit();
     if (limit <= 0) return FIM_ERR_CUDA;
-    TileShape ts;
-    // the bracket's features and labels depend on the tile geometry, so training rows and the
-    // learned launches take the large-image shapes whatever the image size
-    const PlanUse use{(k->n - 1) / 2};
-    fim_status s = choose_tile(k, dtype, use, limit, &ts, 0, 0, 0, true);
-    if (s != FIM_OK) return s;
-    // (r = 64 on 128 rows, whose box of 256 rows takes 16-bit coordinates)
-    if (samples != nullptr && k->shape == kShapeDisk && k->ymax - k->ymin == 128) ts = TileShape{64, 128, 8, 2};
     Plan* p = new (std::nothrow) Plan;
     if (!p) return FIM_ERR_OOM;
-    s = make_plan(k, dtype, use, w, h, ts, limit, p);
+    fim_status s = bracket_plan(k, dtype, w, h, limit, p);
     if (s == FIM_OK) {
-        p->codes = 0;  // the features are values at exact ranks
         p->in = in;
         p->out = out;
         p->pitch = (long long)pitch;

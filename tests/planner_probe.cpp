@@ -52,6 +52,11 @@ fim_status batch_class_k4(const BatchClass& c, const BatchClassArgs* a, int* occ
 }  // namespace fim
 
 extern "C" {
+// The plan of a learned launch or of training rows, kept like a launch's.
+int probe_bracket(const fim_kernel* k, int dtype, int w, int h) {
+    return bracket_plan(k, dtype, w, h, device_smem_limit(), &g_plan);
+}
+
 // A field of the last launch's plan.
 long long probe(const char* f) {
     const Plan& p = g_plan;

@@ -132,3 +132,18 @@ def test_disk_of_256_box_rows_keeps_8_bit_coordinates(lib, monkeypatch):
         assert radii(lib, dtype, 2000, 1500, (30, 64)) == 0
         assert plan(lib, "wide") == [1]
     lib.fim_destroy_kernel(k)
+
+
+@pytest.mark.parametrize("dtype,r,tile", [
+    (U8, 64, (64, 128)), (U16, 64, (64, 128)), (F32, 64, (64, 128)), (U16, 16, (32, 32)), (U16, 48, (64, 128)),
+    (F32, 86, (64, 128)), (F32, 89, (64, 128)), (U8, 89, (64, 128)), (U8, 113, (64, 128)), (U16, 113, (64, 128)),
+    (U16, 114, (64, 64)), (F32, 128, (64, 64))])
+def test_tile_of_the_learned_bracket(lib, dtype, r, tile):
+    """The tiles models have been trained on since the bracket exists: they do not follow the default
+    shapes or the layout of a plan."""
+    k = disk(lib, r)
+    for size in ((300, 200), (4096, 4096)):
+        assert lib.probe_bracket(k, dtype, *size) == 0
+        assert tuple(plan(lib, "Tx", "Ty")) == tile
+        assert plan(lib, "codes") == [0]
+    lib.fim_destroy_kernel(k)
