@@ -319,7 +319,7 @@ fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, 
     if (!p->s16 && !exact_ranks && N <= (1 << 20)) {
         const int base = std::max(0, rank - 1);
         const int64_t top = N - k->n + rank_hi - base;  // the highest feasible rank, relative to base
-        if (top < kMaxSignedRank) {
+        if (top < kMaxSignedRank && !use.full_ranks) {
             p->rank_base = base;
             p->s16 = 1;
             p->rel_max = kMaxSignedRank;
@@ -944,10 +944,12 @@ fim_status choose_tile(const fim_kernel* k, int dtype, const PlanUse& use, int s
 }
 
 // The bracket's features, labels and calibrated width depend on the tile, so training rows and learned
-// launches take the same one, the large-image shape whatever the image size. The sort is exact: the
-// features are values and ranks at places of the sorted footprint.
+// launches take the same one, the large-image shape whatever the image size. The sort is exact and the
+// ordinal image holds whole ranks: the features are values and ranks at places of the sorted footprint
+// (relative and clamped to 15 bits, the ranks at u16 r = 48 lost the lowest 3605 of 33644).
 fim_status bracket_plan(const fim_kernel* k, int dtype, int w, int h, int smem_limit, Plan* p) {
     PlanUse use{(k->n - 1) / 2};
+    use.full_ranks = true;
     use.codes = false;
     TileShape ts;
     const fim_status s = choose_tile(k, dtype, use, smem_limit, &ts, 0, 0, 0, true);

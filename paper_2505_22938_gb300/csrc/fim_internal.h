@@ -225,6 +225,7 @@ struct PlanUse {
     bool exact_ranks = false;  // targets vary per pixel or per kernel: the ordinal image must hold exact
                                // ranks (footprints up to 65535 pixels); otherwise larger footprints
                                // hold ranks relative to the feasible ones of rank .. rank_hi
+    bool full_ranks = false;   // ranks as 16 bits hold them: exact up to 65535 pixels, relative beyond
     bool codes = true;         // the omnigram may be sorted by equalised codes
     // words of further tables in shared memory (several radii): their sum, and their tables of one
     // word per box row

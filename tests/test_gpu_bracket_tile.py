@@ -48,3 +48,30 @@ def test_r64_rows_and_launches_share_a_tile(dtype):
     assert fim.fim_sync_status() == 0
     assert_bit_exact(to_host(out), exp, "learned launch")
     assert int(stats[0]) == seeds
+
+
+def test_rank_features_of_a_large_footprint():
+    """r = 48: a 64 x 128 tile's footprint has 33644 pixels, more than 15 bits of ranks. The last nine
+    features are the ranks, over the footprint's size, of the 3 x 3 pixels at the seed's centre."""
+    import paper_2505_22938_gb300 as fim
+    r, h, w = 48, 128, 64  # one tile
+    img = np.random.default_rng(48).permutation(h * w).reshape(h, w).astype(np.float32)
+    rows, _ = collect(img, "f32", fim.fim_create_kernel_circle(r))
+    half = [int(np.floor(np.sqrt(r * r - dy * dy))) for dy in range(-r, r + 1)]
+    values = []
+    for y in range(-r, h + r):  # row y of the footprint: the widest kernel row that reaches it
+        reach = max(half[y - t + r] for t in range(h) if abs(y - t) <= r)
+        xs = np.clip(np.arange(-reach, w + reach), 0, w - 1)
+        values.append(img[min(max(y, 0), h - 1), xs])
+    values = np.sort(np.concatenate(values))
+    n = len(values)
+    assert n == 33644
+    want = {}
+    for band in range(8):
+        for s in (16, 48):
+            box = img[16 * band + 7:16 * band + 10, s - 1:s + 2].ravel()
+            want[(band, s)] = (np.searchsorted(values, box, "left"), np.searchsorted(values, box, "right"))
+    assert len(rows) == len(want)
+    for row in rows:
+        ranks = np.rint(row[32:41].astype(np.float64) * n)
+        assert any(np.all((lo <= ranks) & (ranks < hi)) for lo, hi in want.values()), ranks

@@ -147,3 +147,15 @@ def test_tile_of_the_learned_bracket(lib, dtype, r, tile):
         assert tuple(plan(lib, "Tx", "Ty")) == tile
         assert plan(lib, "codes") == [0]
     lib.fim_destroy_kernel(k)
+
+
+@pytest.mark.parametrize("dtype", [U8, U16, F32])
+def test_ranks_of_the_learned_bracket(lib, dtype):
+    """Its features are ranks over the footprint's size: whole up to 65535 pixels, 16 bits beyond."""
+    for r in range(8, 129, 4):
+        k = disk(lib, r)
+        assert lib.probe_bracket(k, dtype, 4096, 4096) == 0
+        n, base, top = plan(lib, "N", "rank_base", "rel_max")
+        assert base == 0 if n <= 65535 else base > 0, r
+        assert top >= min(n - 1, 65535), r
+        lib.fim_destroy_kernel(k)
