@@ -685,8 +685,16 @@ fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int 
     const int extent = std::max(k->xmax - k->xmin, k->ymax - k->ymin) + 1;
     const int pw = w > 0 ? w : 1, ph = h > 0 ? h : 1;
     auto valid = [&](const TileShape& c) {
-        return make_plan(k, dtype, use, pw, ph, c, smem_limit, p, cta_threads) == FIM_OK &&
-               p->smem_bytes <= smem_limit && p->shape == k->shape && (!fits || fits(*p));
+        auto planned = [&](const PlanUse& u) {
+            return make_plan(k, dtype, u, pw, ph, c, smem_limit, p, cta_threads) == FIM_OK &&
+                   p->smem_bytes <= smem_limit && p->shape == k->shape;
+        };
+        if (!planned(use)) return false;
+        if (!fits || fits(*p)) return true;
+        if (p->codes == 0) return false;
+        PlanUse exact = use;  // (a sort by codes keeps the radix keys in global scratch)
+        exact.codes = false;
+        return planned(exact) && fits(*p);
     };
     // Waves of the image's tiles on the resident CTAs of the plan in *p (a batch or an unknown size
     // counts as large).
@@ -802,7 +810,7 @@ fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int 
     };
     if (takes(64, 1) || takes(72, 1) || takes(80, 1) || takes(64, 3)) return FIM_OK;
     if (cheapest(std::max(3.0, 0.9 * (extent - 193)), true, 64, false, false)) return FIM_OK;
-    static const TileShape last[] = {{32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}};
+    static const TileShape last[] = {{32, 64, 8, 2}, {32, 32, 8, 2}, {32, 16, 8, 2}, {32, 16, 4, 2}};
     for (const TileShape& c : last)
         if (valid(c)) {
             *ts = c;

@@ -241,8 +241,8 @@ fim_status bracket_plan(const fim_kernel* k, int dtype, int w, int h, int smem_l
 // Tile shape for an image of w x h (w or h <= 0: a batch, which fills the GPU like a large image).
 fim_status choose_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, TileShape* ts, int w,
                        int h, int cta_threads = 0, bool fixed_geometry = false);
-// The untuned tile shape. `fits` (may be null) is one more condition on a candidate's plan; p is
-// storage for trial plans.
+// The untuned tile shape. `fits` (may be null) is one more condition on a candidate's plan, which a plan
+// without a sort by codes may meet in its place; p is storage for trial plans.
 fim_status default_tile(const fim_kernel* k, int dtype, const PlanUse& use, int smem_limit, int w, int h,
                         int cta_threads, bool (*fits)(Plan&), Plan* p, TileShape* ts);
 int device_smem_limit();

@@ -54,7 +54,7 @@ bool fits_array(fim::Plan& p) {
 // the autotuner's cache, whose lookup allocates. Trial plans and the chosen one are built in the
 // caller's storage.
 fim_status pick_plan(const fim_kernel* k, int dtype, int w, int h, int limit, fim::Plan* plan) {
-    const fim::PlanUse use{(k->n - 1) / 2};
+    fim::PlanUse use{(k->n - 1) / 2};
     fim::TileShape ts, small;
     // the library's small-image rule, where its shape also fits the array
     if (fim::default_tile(k, dtype, use, limit, 0, 0, 0, nullptr, plan, &ts) == FIM_OK &&
@@ -64,6 +64,9 @@ fim_status pick_plan(const fim_kernel* k, int dtype, int w, int h, int limit, fi
         return FIM_OK;
     fim_status s = fim::default_tile(k, dtype, use, limit, w, h, 0, fits_array, plan, &ts);
     if (s != FIM_OK) return s;
+    s = fim::make_plan(k, dtype, use, w, h, ts, limit, plan);
+    if (s != FIM_OK || fits_array(*plan)) return s;
+    use.codes = false;
     return fim::make_plan(k, dtype, use, w, h, ts, limit, plan);
 }
 

@@ -159,3 +159,26 @@ def test_ranks_of_the_learned_bracket(lib, dtype):
         assert base == 0 if n <= 65535 else base > 0, r
         assert top >= min(n - 1, 65535), r
         lib.fim_destroy_kernel(k)
+
+
+def noalloc(lib, k, dtype, w, h):
+    return lib.fim_median_noalloc(ctypes.c_void_p(IN), ctypes.c_void_p(OUT), w, h, ctypes.c_size_t(w << dtype), dtype,
+                                  k, 0, None)
+
+
+def test_noalloc_keeps_its_tiles_and_its_calls(lib):
+    """A float tile whose plan by codes does not fit the fixed workspace is planned without codes; spans
+    kernels whose membership table leaves no room for a 512-thread tile take a 256-thread one."""
+    for r in range(41, 61):
+        k = disk(lib, r)
+        assert noalloc(lib, k, F32, 4096, 4096) == 0
+        assert plan(lib, "Tx", "Ty", "codes", "spilled") == [32, 64, 0, 0], r
+        lib.fim_destroy_kernel(k)
+    k = ellipse(lib, 104, 52)
+    for dtype in (U8, U16, F32):
+        for size in ((512, 512), (1537, 1021), (4096, 4096)):
+            assert noalloc(lib, k, dtype, *size) == 0
+    lib.fim_destroy_kernel(k)
+    k = disk(lib, 100)
+    assert noalloc(lib, k, F32, 4096, 4096) == 2  # beyond the workspace, as its test says
+    lib.fim_destroy_kernel(k)
