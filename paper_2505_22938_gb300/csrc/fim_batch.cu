@@ -45,7 +45,11 @@ int esize(int dtype) { return dtype == FIM_U8 ? 1 : (dtype == FIM_U16 ? 2 : 4); 
 // Relative cost of one tile, used only to start the expensive tiles first.
 double tile_cost(const Plan& p) {
     const double px = (double)p.Tx * p.Ty;
-    const double sort = p.sort == kSortRadix ? 12.0 : (p.sort == kSortRadix16 ? 8.0 : (p.sort == kSortCount16x2 ? 6.0 : 3.0));
+    const double sort = p.codes > 0 ? 4.0
+                        : p.sort == kSortRadix ? 12.0
+                        : p.sort == kSortRadix16 ? 8.0
+                        : p.sort == kSortCount16x2 ? 6.0
+                                                   : 3.0;
     return p.N * sort + px * (2.0 * p.ncols + 80.0) + (double)p.RB * p.G * p.n * 2.0;
 }
 
@@ -118,6 +122,7 @@ fim_status fim_batch_create(const fim_job* jobs, int count, fim_batch** out) {
         const fim_job& j = jobs[i];
         const int n = j.kernel->n;
         PlanUse use{(n - 1) / 2};
+        use.fixed_smem = kBatchStaticSmem;
         if (j.percentile >= 0.0) use.rank = std::min(std::max((int)(j.percentile / 100.0 * (n - 1) + 0.5), 0), n - 1);
         TileShape ts;
         // a batch fills the GPU with the tiles of all its jobs: the shapes tuned for large images
@@ -132,9 +137,12 @@ fim_status fim_batch_create(const fim_job* jobs, int count, fim_batch** out) {
         p.ntiles = p.tiles_x * p.tiles_y;
         attach_tma(p);  // the class kernels stage interior footprints like the single-image kernel
     }
-    // classes: the instantiation a plan runs on and its CTA size
+    // Classes: the instantiation a plan runs on, its CTA size, and its resident CTAs per SM up to five: a
+    // class runs at the residency of its largest plan, and one plan of a single CTA would take a second
+    // from all the others (one more or less of six to eight is not worth a launch).
     auto key = [&](const Plan& p) {
-        return std::make_tuple(p.dtype, p.shape, p.wide, p.loc_om < 0 ? 1 : 0, p.scan_groups == 4 ? 4 : 8, p.threads);
+        return std::make_tuple(p.dtype, p.shape, p.wide, p.loc_om < 0 ? 1 : 0, p.scan_groups == 4 ? 4 : 8, p.threads,
+                               std::min(resident_ctas(p), 5));
     };
     std::vector<int> order((size_t)count);
     std::iota(order.begin(), order.end(), 0);

@@ -252,6 +252,7 @@ fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, 
     const bool exact_ranks = use.exact_ranks;
     memset(p, 0, sizeof(*p));
     p->dtype = dtype;
+    p->fixed_smem = use.fixed_smem;
     p->w = w;
     p->h = h;
     p->Tx = ts.Tx;
@@ -516,7 +517,7 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
         // Plans of smaller CTAs that sort by codes take the radix sort for a few tiles only: its keys
         // and list A stay in global scratch, so that the SM holds as many CTAs as its registers allow.
         const bool lean = p->codes > 0 && p->sort == kSortRadix;  // (not changed by the fallback below)
-        const int share = device_smem_per_sm() / std::max(1, 65536 / (p->threads * 64)) / 128 * 128 - 1024;
+        const int share = device_smem_per_sm() / std::max(1, 65536 / (p->threads * 64)) / 128 * 128 - 1024 - p->fixed_smem;
         int mode = 0;
         for (;;) {
             const size_t bins_bytes = p->sort == kSortRadix16 ? 32768 * 4 : 0;
@@ -615,7 +616,7 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
         const int per_sm = device_smem_per_sm();
         auto ctas = [&](size_t bytes) {  // resident CTAs per SM by shared memory and registers
             const int by_regs = 65536 / (p->threads * 64);
-            return per_sm > 0 ? std::min(by_regs, per_sm / (int)(align16(bytes) + 1024)) : 0;
+            return per_sm > 0 ? std::min(by_regs, per_sm / (int)((align16(bytes) + 1024 + p->fixed_smem + 127) / 128 * 128)) : 0;
         };
         if (bw <= 256 && p->SH <= 256 && end <= (size_t)smem_limit && per_sm > 0 && ctas(end) >= ctas(smem) &&
             ctas(end) >= 1) {
@@ -633,11 +634,11 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
 }
 
 // CTAs of a plan resident per SM: its threads at 64 registers each (the kernels' cap), its
-// shared memory plus the 1 KiB the runtime reserves per CTA.
-static int resident_ctas(const Plan& p) {
+// shared memory, the kernel's own and the 1 KiB the runtime reserves per CTA, in units of 128 bytes.
+int resident_ctas(const Plan& p) {
     const int per_sm = device_smem_per_sm();
     const int by_regs = 65536 / (p.threads * 64);
-    const int by_smem = per_sm > 0 ? per_sm / (p.smem_bytes + 1024) : 1;
+    const int by_smem = per_sm > 0 ? per_sm / ((p.smem_bytes + 1024 + p.fixed_smem + 127) / 128 * 128) : 1;
     return std::max(1, std::min(std::min(by_regs, by_smem), std::min(2048 / p.threads, 32)));
 }
 

@@ -171,12 +171,18 @@ struct Plan {
     int spans[kMaxExtent];                // per row i: (lo & 0xffff) | (hi << 16)
     // tensor map of the input image for the footprint copies (valid when use_tma)
     CUtensorMap tmap;  // (the type carries the alignment the copies need)
+    int fixed_smem;    // host: static shared memory of the kernel the plan is made for
 };
 
 // Bytes of a Plan before its tables: all the tile pipeline reads once the tables are in
 // shared memory.
 constexpr size_t kPlanScalarBytes = ((offsetof(Plan, frow) + 15) / 16) * 16;
 static_assert(offsetof(Plan, frow) % 4 == 0, "plan scalars are copied as 32-bit words");
+
+// Static shared memory of a single-image kernel and of a batch class kernel (which holds the current
+// plan's scalars), with the gap before the dynamic part's 128-byte alignment.
+constexpr int kLaunchStaticSmem = 128;
+constexpr int kBatchStaticSmem = (int)((kPlanScalarBytes + 32 + 127) / 128 * 128);
 
 
 // One class of a batch: jobs whose plans run on the same tile-pipeline instantiation and CTA size.
@@ -227,12 +233,15 @@ struct PlanUse {
                                // hold ranks relative to the feasible ones of rank .. rank_hi
     bool full_ranks = false;   // ranks as 16 bits hold them: exact up to 65535 pixels, relative beyond
     bool codes = true;         // the omnigram may be sorted by equalised codes
+    int fixed_smem = kLaunchStaticSmem;  // static shared memory of the kernel
     // words of further tables in shared memory (several radii): their sum, and their tables of one
     // word per box row
     int table_words = 0, row_tables = 0;
 };
 fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, int h, const TileShape& ts,
                      int smem_limit, Plan* p, int cta_threads = 0);
+// CTAs of the plan resident per SM.
+int resident_ctas(const Plan& p);
 // Re-lays out a plan whose model is set so that the bracket MLP's parameters are staged in
 // shared memory; keeps them in device memory (off_model = -1) when they do not fit.
 fim_status plan_stage_model(Plan* p, int smem_limit);

@@ -57,6 +57,19 @@ int probe_bracket(const fim_kernel* k, int dtype, int w, int h) {
     return bracket_plan(k, dtype, w, h, device_smem_limit(), &g_plan);
 }
 
+// Resident CTAs per SM of the class of the given jobs and threads in the last batch (0: no such class).
+int probe_class(int dtype, int threads, int jobs) {
+    int ctas = 0;
+    for (size_t i = 0; i < g_classes.size(); ++i)
+        if (g_classes[i].dtype == dtype && g_classes[i].threads == threads && g_classes[i].njobs == jobs)
+            ctas = g_class_ctas[i];
+    return ctas;
+}
+void probe_forget_classes() {
+    g_classes.clear();
+    g_class_ctas.clear();
+}
+
 // A field of the last launch's plan.
 long long probe(const char* f) {
     const Plan& p = g_plan;

@@ -182,3 +182,34 @@ def test_noalloc_keeps_its_tiles_and_its_calls(lib):
     k = disk(lib, 100)
     assert noalloc(lib, k, F32, 4096, 4096) == 2  # beyond the workspace, as its test says
     lib.fim_destroy_kernel(k)
+
+
+class Job(ctypes.Structure):
+    _fields_ = [("src", ctypes.c_void_p), ("dst", ctypes.c_void_p), ("w", ctypes.c_int), ("h", ctypes.c_int),
+                ("pitch", ctypes.c_size_t), ("dtype", ctypes.c_int), ("kernel", ctypes.c_void_p),
+                ("percentile", ctypes.c_double)]
+
+
+def batch(lib, dtype, rs):
+    jobs = (Job * len(rs))()
+    for i, r in enumerate(rs):
+        jobs[i] = Job((1 << 40) + (i << 32), (1 << 42) + (i << 32), 1000, 900, 1000 << dtype, dtype, disk(lib, r).value,
+                      -1.0)
+    b = ctypes.c_void_p()
+    lib.probe_forget_classes()
+    assert lib.fim_batch_create(jobs, len(rs), ctypes.byref(b)) == 0
+
+
+def test_batch_classes_keep_the_residency_of_their_tiles(lib):
+    """The class kernels' static shared memory is part of a batch's plans, and a plan of fewer resident
+    CTAs has a class of its own."""
+    batch(lib, F32, [18, 30, 42, 45, 49])
+    assert lib.probe_class(F32, 512, 5) == 2
+    batch(lib, U16, [24, 28])
+    assert lib.probe_class(U16, 512, 2) == 2
+    batch(lib, U8, [36, 42, 53, 57, 95, 96])
+    assert lib.probe_class(U8, 512, 4) == 2 and lib.probe_class(U8, 512, 2) == 1
+    batch(lib, F32, [15, 16])
+    assert lib.probe_class(F32, 256, 2) == 4
+    batch(lib, U8, [2, 4, 8, 12, 16])  # six to eight CTAs: one class
+    assert lib.probe_class(U8, 128, 5) >= 6
