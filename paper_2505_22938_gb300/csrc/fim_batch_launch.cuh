@@ -68,8 +68,10 @@ template <int DT, int SHAPE, int W, int OG, int KS>
 fim_status batch_class_typed(const BatchClassArgs* a, int threads, int smem, int* occ, cudaStream_t stream,
                              int grid) {
     auto fn = batch_class_kernel<DT, SHAPE, W, OG, KS>;
-    if (a == nullptr) {  // set-up: shared-memory opt-in and the resident CTAs per SM
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+    if (a == nullptr) {
+        // Set-up: shared-memory opt-in and the resident CTAs per SM. The opt-in is the function's, not the
+        // batch's: always to the device's limit, so that a batch of smaller plans leaves it to the others.
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, device_smem_limit()) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, fn, threads, smem) != cudaSuccess) {
             cudaGetLastError();
             return FIM_ERR_CUDA;
