@@ -1540,7 +1540,8 @@ __device__ __forceinline__ float bf16_to_f32(uint16_t b) { return __uint_as_floa
 
 // Features of the seed window centred at box position (cu, cv): the tile's normalised value
 // quantiles (already in q[0..31]) and the ranks / N of the 3x3 pixels around the centre
-// (the centre's own rank where a neighbour lies outside the footprint).
+// (the centre's own rank where a neighbour lies outside the footprint, 0 where the centre does: a
+// kernel may lie off its centre).
 __device__ __forceinline__ void seed_features(const uint16_t* ord, int SP, const int* frow, int SH, int N, int cu,
                                               int cv, const float* q, float* fa, float* fb) {
     const int lane = threadIdx.x & 31;
@@ -1556,8 +1557,13 @@ __device__ __forceinline__ void seed_features(const uint16_t* ord, int SP, const
         if (!in) {
             u = cu;
             v = cv;
+            in = v >= 0 && v < SH;
+            if (in) {
+                const int fr = frow[v];
+                in = u >= span_lo(fr) && u <= span_hi(fr);
+            }
         }
-        nb = (float)ord[v * SP + u] / (float)N;
+        nb = in ? (float)ord[v * SP + u] / (float)N : 0.f;
     }
     *fb = nb;
 }
@@ -2091,7 +2097,10 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
     #pragma unroll
             for (int q = 0; q < kRowsPerLane; ++q) {
                 const int i = lane + 32 * q;
-                eo[q] = lo[q] = 0;  // rows beyond the kernel compare the centre with itself: no change
+                // rows beyond the kernel compare a pixel of the window with itself: no change (not the
+                // centre, which lies outside the footprint, and may lie outside shared memory, where
+                // the kernel is off centre)
+                eo[q] = lo[q] = qhtab[0].x;
                 if (i < qnrows) {
                     const int2 o = qhtab[i];
                     eo[q] = right ? o.y : o.x - 1;
