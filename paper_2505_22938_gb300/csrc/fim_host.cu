@@ -1478,7 +1478,9 @@ fim_status fim_median_host(const void* in_host, void* out_host, int w, int h, si
         for (int b = 0; b < bands && s == FIM_OK; ++b) {
             const int tr0 = b * rows_per_band, tr1 = std::min(p->tiles_y, tr0 + rows_per_band);
             const int y0 = tr0 * p->Ty, y1 = std::min(h, tr1 * p->Ty);
-            const int need = std::min(h, y1 + p->ymax);  // rows [0, need) feed this band
+            // rows [0, need) feed this band; rows above the image repeat row 0, which a kernel that lies
+            // above its centre may need alone
+            const int need = std::min(h, std::max(1, y1 + p->ymax));
             if (need > copied) {
                 if (cudaMemcpy2DAsync((void*)(din + (size_t)copied * dpitch), dpitch,
                                       hin + (size_t)copied * pitch_bytes, pitch_bytes, dpitch, need - copied,
