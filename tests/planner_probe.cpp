@@ -85,6 +85,14 @@ long long probe(const char* f) {
     if (!strcmp(f, "feasible")) return p.N - p.n + p.rank - p.rank_base;  // highest, as stored
     if (!strcmp(f, "wide")) return p.wide;
     if (!strcmp(f, "sort")) return p.sort;
+    if (!strcmp(f, "inside")) {  // tiles whose box lies inside the image
+        int n = 0;
+        for (int t = 0; t < p.tiles_x * p.tiles_y; ++t) {
+            const int x = t % p.tiles_x * p.Tx + p.xmin, y = t / p.tiles_x * p.Ty + p.ymin;
+            n += x >= 0 && y >= 0 && x + p.S <= p.w && y + p.SH <= p.h;
+        }
+        return n;
+    }
     if (!strcmp(f, "resident")) return resident(p.threads, p.smem_bytes, 128);
     abort();
 }

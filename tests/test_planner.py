@@ -213,3 +213,21 @@ def test_batch_classes_keep_the_residency_of_their_tiles(lib):
     assert lib.probe_class(F32, 256, 2) == 4
     batch(lib, U8, [2, 4, 8, 12, 16])  # six to eight CTAs: one class
     assert lib.probe_class(U8, 128, 5) >= 6
+
+
+def test_plans_of_the_codes_tests_sort_by_codes(lib, monkeypatch):
+    """Every plan of test_gpu_codes_interior.py, with at least two tiles whose box lies inside the image."""
+    import numpy as np
+    import test_gpu_codes_interior as t
+    for dtype, spec, tile in t.PLANS:
+        monkeypatch.setenv("FIM_TILE", tile)
+        k = ctypes.c_void_p()
+        if spec[0] == "polygon":
+            xy = np.ascontiguousarray(spec[1], np.float64)
+            assert lib.fim_create_kernel_polygon(xy.ctypes.data_as(ctypes.c_void_p), len(xy), ctypes.byref(k)) == 0
+        else:
+            k = disk(lib, spec[1]) if spec[0] == "circle" else ellipse(lib, *spec[1:])
+        assert median(lib, k, {"u16": U16, "f32": F32}[dtype], t.W, t.H) == 0
+        assert plan(lib, "codes") == [1], spec
+        assert plan(lib, "inside")[0] >= 2, spec
+        lib.fim_destroy_kernel(k)
