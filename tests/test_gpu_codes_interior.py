@@ -28,7 +28,7 @@ def image(kind, dtype):
     if kind == "uniform":  # codes of one to four pixels and a few more
         a = rng.random((H, W)) * 60000.0
     elif kind == "clusters":  # about five pixels within a few units in the last place: one code, different keys
-        a = rng.integers(1, 3000, (H, W)) * (19.0 if dtype == "u16" else 1e3) + rng.integers(0, 3, (H, W)) * (1 if dtype == "u16" else 1e-4)
+        a = rng.integers(1, 3000, (H, W)) * (19.0 if dtype == "u16" else 1e3) + rng.integers(0, 3, (H, W)) * (1 if dtype == "u16" else 0.25)
     elif kind == "one group":  # smooth, but for 40 pixels of neighbouring values in every tile: the exact sort
         a = datagen.image_for("f32", 5, H, W).astype(np.float64)
         if dtype == "u16":
