@@ -194,9 +194,12 @@ def sort_passes(dtype: str, threads: int, footprint: int = 0) -> int:
     """Key passes of the ordinal transform the library runs for a plan (see the docstring above);
     footprints beyond 65535 pixels overflow the 16-bit counters of the 65536-bin pass: 16-bit
     data and the float keys' 16-bit pass count in two rounds of the same pass."""
-    coded = 8000 <= footprint <= 65535  # full CTAs, and smaller ones with enough pixels, sort by codes
+    # float keys in full CTAs, and smaller CTAs with enough pixels, sort by codes
+    if dtype == "f32" and threads >= 1024:
+        return 1 if footprint <= 65535 else 3
+    coded = 8000 <= footprint <= 65535
     if dtype == "f32":
-        return 1 if coded and threads >= 256 else (3 if threads >= 1024 else 4)
+        return 1 if coded and threads >= 256 else 4
     if dtype == "u16" and threads < 1024:
         return 1 if coded and threads >= 512 else 2
     if dtype == "u16" and footprint > 65535:  # the counting sort in two rounds over the key range

@@ -219,10 +219,11 @@ fim_status fim_autotune_clear(void);
  * Batched persistent launch. One job is one 2-D image filtered with its own kernel, dtype, size
  * and pitch; percentile < 0 selects the median, otherwise the percentile filter of fim_percentile.
  * The jobs are grouped into classes by the pipeline they run (dtype, kernel shape, omnigram
- * encoding and home, scan width) and CTA size. Each class is one persistent kernel whose CTAs
- * take tiles from one device-side queue over the tiles of all the class's jobs (expensive tiles
- * first); a class of one job runs the single-image kernel on that job. The classes run side by
- * side on the batch's own streams, forked from and joined to the caller's. Not part of the paper.
+ * encoding and home, kernel set), CTA size and resident CTAs. Each class is one persistent kernel
+ * whose CTAs take tiles from one device-side queue over the tiles of all the class's jobs
+ * (expensive tiles first); a class of one job runs the single-image kernel on that job. The classes
+ * run side by side on the batch's own streams, forked from and joined to the caller's. Not part of
+ * the paper.
  */
 typedef struct {
     const void* in;      /* device pointer */

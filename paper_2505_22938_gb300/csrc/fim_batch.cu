@@ -1,6 +1,6 @@
 // Batched persistent launch (host side): many images of any size, dtype and kernel. The jobs are
-// grouped into classes that share a tile-pipeline instantiation and CTA size; each class runs as
-// one persistent kernel whose device-side queue spans the tiles of all its jobs (sorted by
+// grouped into classes that share a tile-pipeline instantiation, CTA size and resident CTAs; each class
+// runs as one persistent kernel whose device-side queue spans the tiles of all its jobs (sorted by
 // decreasing cost per tile), and the class kernels run side by side on forked streams, so the
 // tail of one class overlaps the others. The batch object owns its device-side plans, queues and
 // workspace and its side streams; fim_batch_run() only zeroes the queue counters and launches,
@@ -141,7 +141,7 @@ fim_status fim_batch_create(const fim_job* jobs, int count, fim_batch** out) {
     // class runs at the residency of its largest plan, and one plan of a single CTA would take a second
     // from all the others (one more or less of six to eight is not worth a launch).
     auto key = [&](const Plan& p) {
-        return std::make_tuple(p.dtype, p.shape, p.wide, p.loc_om < 0 ? 1 : 0, p.scan_groups == 4 ? 4 : 8, p.threads,
+        return std::make_tuple(p.dtype, p.shape, p.wide, p.loc_om < 0 ? 1 : 0, p.kernel_set == 4 ? 4 : 8, p.threads,
                                std::min(resident_ctas(p), 5));
     };
     std::vector<int> order((size_t)count);
@@ -166,7 +166,7 @@ fim_status fim_batch_create(const fim_job* jobs, int count, fim_batch** out) {
             c.shape = p.shape;
             c.wide = p.wide;
             c.og = p.loc_om < 0 ? 1 : 0;
-            c.ks = p.scan_groups == 4 ? 4 : 8;
+            c.ks = p.kernel_set == 4 ? 4 : 8;
             c.threads = p.threads;
             classes.push_back(c);
             first_job.push_back(i);

@@ -386,7 +386,10 @@ fim_status make_plan(const fim_kernel* k, int dtype, const PlanUse& use, int w, 
     // Sort by equalised codes: float keys in full CTAs, and float and 16-bit keys in CTAs of 256
     // threads or more with enough pixels; footprints whose packed 16-bit places and 8-bit
     // coordinates hold. About 1.5 codes per pixel, in units the scan splits evenly (layout_plan
-    // takes fewer where shared memory ends).
+    // takes fewer where shared memory ends). The bounds on the smaller CTAs keep the sort to tiles
+    // that spread its fixed work (up to 3072 table entries cleared and dealt) over enough pixels:
+    // 64x64 tiles gain from f32 r = 14 (8236 pixels) and u16 r = 23 on, u16 r = 8 in 32x32 tiles (2212
+    // pixels) lost (sort 43k -> 85k cycles); what lies between was not measured.
     p->codes = 0;
     const bool lean = use.codes && p->sort == kSortRadix && p->threads < 1024 && p->N >= 8000 && ts.Tx * ts.Ty >= 2048 &&
                       p->threads >= (dtype == FIM_F32 ? 256 : 512);
@@ -564,7 +567,8 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
             auto fitting = [&](size_t bytes) {
                 return bytes < uni + table_bytes ? 0 : (int)std::min<size_t>(p->codes, (bytes - uni - table_bytes) / 2 / unit * unit);
             };
-            // a resident CTA less costs more than a few more pixels per code
+            // (a resident CTA less costs more than a few more pixels per code, down to 0.75 codes per pixel,
+            // half of what is asked for)
             const int shared = lean && uni + solve_bytes <= (size_t)share ? fitting((size_t)share) : 0;
             p->codes = shared >= p->N - p->N / 4 ? shared : fitting((size_t)smem_limit);
             if (p->codes < p->N / 2) p->codes = 0;
@@ -627,7 +631,7 @@ fim_status layout_plan(Plan* p, int smem_limit, bool stage_model) {
     }
     p->smem_bytes = (int)align16(smem);
     p->group_bytes = p->smem_bytes - p->tab_bytes;
-    p->scan_groups = p->threads < 1024 && p->codes == 0 ? 4 : 8;
+    p->kernel_set = p->threads < 1024 && p->codes == 0 ? 4 : 8;
     p->groups = 1;
     p->scratch_per_cta = (long long)glob;
     return FIM_OK;

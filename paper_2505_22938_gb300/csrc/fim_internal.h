@@ -84,7 +84,7 @@ struct Plan {
     int Tx, Ty, txshift, RB, G;
     int threads, nwarps;    // CTA size (all cooperative loops and per-warp buffers)
     int vthreads;           // 2*Tx*RB: threads of the vertical sweep (the first ones of the CTA)
-    int scan_groups;        // kernel set: 8 the 1024-thread CTAs' and the sort by codes, 4 the others (fim_tile_k4.cu)
+    int kernel_set;         // 8: the kernels of 1024-thread CTAs and of the sort by codes, 4: the others (fim_tile_k4.cu)
     int S, SH;              // footprint bounding box (columns, rows)
     int SP;                 // row pitch (elements) of the ordinal image; SP/2 is odd
     int tiles_x, tiles_y;
@@ -188,7 +188,7 @@ constexpr int kBatchStaticSmem = (int)((kPlanScalarBytes + 32 + 127) / 128 * 128
 // One class of a batch: jobs whose plans run on the same tile-pipeline instantiation and CTA size.
 struct BatchClass {
     int dtype, shape, wide, og, ks;  // instantiation: element type, kernel shape, omnigram encoding
-                                     // and home (global when og), scan groups per step (4 or 8)
+                                     // and home (global when og), kernel set (4 or 8)
     int threads, smem;               // CTA size and dynamic shared memory (the largest of its plans)
     int grid;                        // persistent CTAs
     int njobs, total_tiles;
@@ -290,7 +290,7 @@ bool small_image_shape(const fim_kernel* k, int dtype, const PlanUse& use, int w
 fim_status launch_tile_kernel(Plan& p, cudaStream_t stream);
 fim_status read_and_clear_device_status(cudaStream_t stream);
 
-// (fim_tile_k4.cu) the kernels with 4 omnigram groups per scan step, and their status word
+// (fim_tile_k4.cu) the kernels of smaller CTAs, and their status word
 fim_status launch_tile_kernel_k4(Plan& p, cudaStream_t stream);
 fim_status launch_tile_kernel_fixed_k4(Plan& p, unsigned char* scratch, size_t capacity, cudaStream_t stream,
                                        bool launch);

@@ -8,12 +8,12 @@ fim_status launch_tile_kernel(Plan& p, cudaStream_t stream) {
     if (p.rank_map != nullptr) return launch_tile_kernel_map(p, stream);
     if (p.model != nullptr || p.samples != nullptr || p.stats != nullptr || p.nranks > 1 || p.multi)
         return launch_tile_kernel_extras(p, stream);
-    return p.scan_groups == 4 ? launch_tile_kernel_k4(p, stream) : launch_tile_kernel_ks<8>(p, stream);
+    return p.kernel_set == 4 ? launch_tile_kernel_k4(p, stream) : launch_tile_kernel_ks<8>(p, stream);
 }
 
 fim_status launch_tile_kernel_fixed(Plan& p, unsigned char* scratch, size_t capacity, cudaStream_t stream,
                                     bool launch) {
-    return p.scan_groups == 4 ? launch_tile_kernel_fixed_k4(p, scratch, capacity, stream, launch)
+    return p.kernel_set == 4 ? launch_tile_kernel_fixed_k4(p, scratch, capacity, stream, launch)
                               : launch_tile_kernel_fixed_ks<8>(p, scratch, capacity, stream, launch);
 }
 

@@ -8,7 +8,7 @@ namespace fim {
 fim_status launch_tile_kernel_extras(Plan& p, cudaStream_t stream) {
     // the 1024-thread tiles of large kernels (where the learned bracket is meant to help) get a
     // set of their own; other plans share one
-    return p.scan_groups == 8 ? launch_tile_kernel_ks<8, 1>(p, stream) : launch_tile_kernel_ks<0, 1>(p, stream);
+    return p.kernel_set == 8 ? launch_tile_kernel_ks<8, 1>(p, stream) : launch_tile_kernel_ks<0, 1>(p, stream);
 }
 
 fim_status read_and_clear_extras_status() { return read_and_clear_unit_status(); }

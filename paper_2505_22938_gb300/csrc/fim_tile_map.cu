@@ -6,7 +6,7 @@
 namespace fim {
 
 fim_status launch_tile_kernel_map(Plan& p, cudaStream_t stream) {
-    return p.scan_groups == 8 ? launch_tile_kernel_ks<8, 2>(p, stream) : launch_tile_kernel_ks<0, 2>(p, stream);
+    return p.kernel_set == 8 ? launch_tile_kernel_ks<8, 2>(p, stream) : launch_tile_kernel_ks<0, 2>(p, stream);
 }
 
 fim_status read_and_clear_map_status() { return read_and_clear_unit_status(); }

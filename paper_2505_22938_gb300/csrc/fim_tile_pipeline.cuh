@@ -8,11 +8,14 @@
 //                          8-bit, and 16-bit data in 1024-thread CTAs: counting sort over 256 /
 //                                         65536 shared-memory bins, the bucket construction of
 //                                         Eq. 5 run by all threads;
-//                          float in 1024-thread CTAs: counting sort by equalised 16-bit codes,
-//                                         ties settled at the output;
+//                          float in 1024-thread CTAs, and float and 16-bit data in the 256- and
+//                                         512-thread CTAs of larger tiles, where the tile's box
+//                                         lies inside the image: counting sort by equalised
+//                                         16-bit codes, ties settled at the output;
 //                          float otherwise, and 16-bit data in smaller CTAs: LSD radix sort of
-//                                         order-preserving keys (Sec. 4.1 float key), 8-bit
-//                                         passes (four / two).
+//                                         order-preserving keys (Sec. 4.1 float key): for float in
+//                                         1024-thread CTAs with room for its bins a 16-bit and
+//                                         two 8-bit passes, else 8-bit passes (four / two).
 //   2. ordinal image   - I(Omega[v]) = v (Eq. 4), exact 16-bit ranks.
 //   3. seed solve      - RB*G seed windows, one warp each: coarse histogram of I over the
 //                        window, then a ballot scan of Omega to the exact median (Sec. 4.2).
@@ -949,7 +952,7 @@ __device__ void ordinal_transform_count(const Plan& P, const int* frow, uint32_t
 // ---- ordinal transform by equalised codes --------------------------------------------------
 // Float keys have no counting sort of their own size, and an LSD radix sort's stable passes cost a
 // warp match per 32 pixels (64 cycles of the SM where the digits differ) and a scattered global
-// store. In full CTAs one counting sort places every pixel by a 16-bit code that follows the
+// store. In CTAs of 256 threads or more one counting sort places every pixel by a 16-bit code that follows the
 // tile's own distribution instead: histograms of a sample of the footprint over the keys' top bits
 // deal out codes in proportion, in two levels so that a tile whose values differ in their low
 // bits only is resolved as well, and within one bin the code is linear in the key. Codes never
@@ -1802,9 +1805,9 @@ __device__ __forceinline__ void process_tile(const Plan& P, int tile, unsigned c
             }
         }
     }
-    // float data always takes the radix sort; 16-bit data takes it in small CTAs, where the
-    // counting sort's 65536 bins would keep other CTAs off the SM
-    // the sort, compiled for the staged box and for the image (one branch per tile)
+    // The sort, compiled for the staged box and for the image (one branch per tile): by codes where the
+    // plan has them and the box lies inside the image; otherwise float data takes the radix sort, and
+    // 16-bit data in small CTAs, where the counting sort's 65536 bins would keep other CTAs off the SM.
     auto sort = [&](auto staged) {
         constexpr bool ST = decltype(staged)::value;
         if constexpr (kCodes) {
